@@ -873,23 +873,47 @@ static sdp_status sytrd(cudaStream_t st, int n, double* A, EigWork* w) {
 // which matters on GB300 where every FP64 op of a warp costs many cycles; the
 // sequence is rescaled by a power of two every 16 steps to stay in range.
 // A zero minor takes the sign opposite to its predecessor.
+// Three FP64 instructions a step and nothing else on that pipe: signs, the zero
+// test and the range test are integer tests on the bits (an FP64 compare takes
+// the pipe as long as a multiply-add; with them the step took 3.6 times as long).
+__device__ __forceinline__ bool sturm_neg(double p, bool before) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(p) << 1;
+  // zero or NaN: the sign opposite to the predecessor's
+  return (u - 1ull >= 0xFFE0000000000000ull) ? !before : __double2hiint(p) < 0;
+}
 __device__ __forceinline__ int sturm_count(int n, const double* d, const double* e2, double x) {
   double pm = 1.0, p = d[0] - x;
-  int sp = (p > 0.0) ? 1 : -1;       // sign of p_0 = 1 is +1; zero counts as a change
-  int cnt = (sp < 0) ? 1 : 0;
-  for (int i = 1; i < n; ++i) {
-    const double pn = fma(d[i] - x, p, -e2[i - 1] * pm);
-    const int sn = (pn > 0.0) ? 1 : (pn < 0.0 ? -1 : -sp);
-    cnt += (sn != sp);
-    sp = sn;
+  bool neg = !(p > 0.0);             // sign of p_0 = 1 is +1; zero counts as a change
+  int cnt = neg ? 1 : 0;
+  int i = 1;
+  auto step = [&](int t) {
+    const double pn = fma(d[t] - x, p, -e2[t - 1] * pm);
+    const bool sn = sturm_neg(pn, neg);
+    cnt += (sn != neg) ? 1 : 0;
+    neg = sn;
     pm = p;
     p = pn;
-    if ((i & 15) == 0) {
-      const double a = fmax(fabs(p), fabs(pm));
-      if (a > 0x1p+400) { p *= 0x1p-400; pm *= 0x1p-400; }
-      else if (a < 0x1p-400 && a > 0.0) { p *= 0x1p+400; pm *= 0x1p+400; }
-    }
+  };
+  auto rescale = [&]() {
+    const unsigned long long m = 0x7FFFFFFFFFFFFFFFull;
+    const unsigned long long up = (unsigned long long)__double_as_longlong(p) & m;
+    const unsigned long long um = (unsigned long long)__double_as_longlong(pm) & m;
+    const unsigned long long ua = up > um ? up : um;
+    if (ua > 0x58F0000000000000ull) { p *= 0x1p-400; pm *= 0x1p-400; }                     // above 2^400
+    else if (ua < 0x26F0000000000000ull && ua > 0ull) { p *= 0x1p+400; pm *= 0x1p+400; }   // below 2^-400
+  };
+  for (; i < n && (i & 15) != 0; ++i) step(i);
+  if (i < n) {
+    step(i);
+    rescale();
+    ++i;
   }
+  for (; i + 15 < n; i += 16) {
+#pragma unroll
+    for (int u = 0; u < 16; ++u) step(i + u);
+    rescale();
+  }
+  for (; i < n; ++i) step(i);        // fewer than 16 left: no multiple of 16 among them
   return cnt;
 }
 
@@ -906,35 +930,66 @@ __device__ void gersh(int n, const double* d, const double* e, double* lo, doubl
   *hi = gu + pad;
 }
 
-// Stage d and e^2 in shared memory (2n doubles) and compute Gershgorin bounds.
-__device__ void stage_tri(int n, const double* d, const double* e, double* sd, double* se2, double* s_lo,
-                          double* s_hi) {
+// Gershgorin bounds of a tridiagonal by the whole block (minima and maxima do
+// not depend on the order); red: 2 x 32 doubles of shared memory.
+__device__ void gersh_block(int n, const double* d, const double* e, double* red, double* lo, double* hi) {
+  double gl = d[0], gu = d[0];
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    sd[i] = d[i];
-    se2[i] = (i + 1 < n) ? e[i] * e[i] : 0.0;
+    const double r = (i > 0 ? fabs(e[i - 1]) : 0.0) + (i + 1 < n ? fabs(e[i]) : 0.0);
+    gl = fmin(gl, d[i] - r);
+    gu = fmax(gu, d[i] + r);
   }
-  if (threadIdx.x == 0) gersh(n, d, e, s_lo, s_hi);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    gl = fmin(gl, __shfl_xor_sync(0xffffffffu, gl, o));
+    gu = fmax(gu, __shfl_xor_sync(0xffffffffu, gu, o));
+  }
+  if ((threadIdx.x & 31) == 0) {
+    red[threadIdx.x >> 5] = gl;
+    red[32 + (threadIdx.x >> 5)] = gu;
+  }
   __syncthreads();
+  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+    gl = fmin(gl, red[w]);
+    gu = fmax(gu, red[32 + w]);
+  }
+  const double tn = fmax(fabs(gl), fabs(gu));
+  const double pad = 2.0 * DBL_EPSILON * tn * n + 4.0 * DBL_MIN;
+  *lo = gl - pad;
+  *hi = gu + pad;
 }
 
 __device__ __forceinline__ bool bis_done(double lo, double hi) {
   return hi - lo <= 2.0 * DBL_EPSILON * fmax(fabs(lo), fabs(hi)) + 4.0 * DBL_MIN;
 }
 
-// w[t] = eigenvalue number idx[t] (ascending, 0-based) of T; one warp per
-// eigenvalue, 32-point multisection per round (five bits per round).
-__global__ void k_stebz(int n, const double* d, const double* e, int cnt, const int* idx, int i0, double* wout) {
+// Eigenvalue number idx[t] (or i0 + t; ascending, 0-based) of T for t < cnt, into
+// wout[t]; with wfirst != nullptr the first one goes there and the rest to
+// wout[0..].  One warp per eigenvalue, 32-point multisection per round (five bits
+// per round).  Serial in n: a round is a chain of n dependent multiply-adds, and
+// about 12 rounds are needed.  Warps that share an SM share its FP64 pipe, so few
+// eigenvalues get one warp per block (wpb = 1; the other warps only stage T).
+// An FP64 warp instruction holds its scheduler's pipe for 64 cycles, so a step costs
+// 192: n = 565, 565 eigenvalues or 5: 1616 us -> 897 us; n = 2000: 9.8 ms -> 7.0 ms.
+__global__ void __launch_bounds__(128) k_stebz(int n, const double* d, const double* e, int cnt, const int* idx,
+                                               int i0, double* wout, double* wfirst, int wpb) {
   extern __shared__ double tri[];
-  __shared__ double s_lo, s_hi;
-  stage_tri(n, d, e, tri, tri + n, &s_lo, &s_hi);
-  const int lane = threadIdx.x % 32;
-  const int t = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
-  if (t >= cnt) return;
+  __shared__ double red[64];
+  double* sd = tri;
+  double* se2 = tri + n;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    sd[i] = d[i];
+    se2[i] = (i + 1 < n) ? e[i] * e[i] : 0.0;
+  }
+  double lo, hi;
+  gersh_block(n, d, e, red, &lo, &hi);   // its barrier also covers the staging
+  const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
+  const int t = blockIdx.x * wpb + warp;
+  if (warp >= wpb || t >= cnt) return;
   const int target = idx ? idx[t] : i0 + t;
-  double lo = s_lo, hi = s_hi;
   for (int round = 0; round < 64 && !bis_done(lo, hi); ++round) {
     const double h = (hi - lo) / 33.0;
-    const int c = sturm_count(n, tri, tri + n, lo + h * (lane + 1));
+    const int c = sturm_count(n, sd, se2, lo + h * (lane + 1));
     const unsigned above = __ballot_sync(0xffffffffu, c > target);
     const int first = above ? __ffs(above) - 1 : 32;
     const double nlo = (first == 0) ? lo : lo + h * first;
@@ -943,7 +998,10 @@ __global__ void k_stebz(int n, const double* d, const double* e, int cnt, const 
     lo = nlo;
     hi = nhi;
   }
-  if (lane == 0) wout[t] = 0.5 * (lo + hi);
+  if (lane == 0) {
+    if (wfirst && t == 0) *wfirst = 0.5 * (lo + hi);
+    else wout[wfirst ? t - 1 : t] = 0.5 * (lo + hi);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -1313,12 +1371,12 @@ int eig_flag(cudaStream_t st, EigWork* w) {
 }
 
 static void launch_stebz(cudaStream_t st, int n, const double* d, const double* e, int cnt, const int* idx,
-                         int i0, double* out) {
+                         int i0, double* out, double* first = nullptr) {
   const size_t smem = 2 * (size_t)n * sizeof(double);
   allow_max_smem((const void*)k_stebz);
-  const int warps = 4;
+  const int wpb = (cnt >= 4 * 148) ? 4 : std::max(1, (int)cdiv(cnt, 148));
   count_launch();
-  k_stebz<<<cdiv(cnt, warps), 32 * warps, smem, st>>>(n, d, e, cnt, idx, i0, out);
+  k_stebz<<<cdiv(cnt, wpb), 128, smem, st>>>(n, d, e, cnt, idx, i0, out, first, wpb);
 }
 
 // Splits T into unreduced blocks; returns the number of blocks (host sync).
@@ -1414,12 +1472,14 @@ sdp_status eig_extremes(cudaStream_t st, int n, double* A, int k, double* lmin_d
   SDP_TRY(sytrd(st, n, A, w));
   const int nb = (k > 0) ? split_blocks(st, n, w) : 1;
   if (nb <= 1) {
-    launch_stebz(st, n, w->d, w->e, 1, nullptr, 0, lmin_dev);
-    if (k == 0) return SDP_OK;
+    if (k == 0) {
+      launch_stebz(st, n, w->d, w->e, 1, nullptr, 0, lmin_dev);
+      return SDP_OK;
+    }
     int* idx = (int*)w->part;  // small scratch (part is idle here)
     count_launch(1);
     k_idx_extremes<<<1, 128, 0, st>>>(n, k, idx);
-    launch_stebz(st, n, w->d, w->e, k, idx + 1, 0, wtop);
+    launch_stebz(st, n, w->d, w->e, k + 1, idx, 0, wtop, lmin_dev);   // the smallest and the top k at once
     eigenvectors(st, n, w, 1, wtop, 0, k, Etop);
   } else {
     eigenvalues_all(st, n, w, nb, w->wsel);
