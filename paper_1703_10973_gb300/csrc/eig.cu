@@ -1140,6 +1140,234 @@ __global__ void k_stein(int nfull, const double* __restrict__ dfull, const doubl
 #undef WS
 }
 
+// The same inverse iteration with the working arrays in shared memory: a block of
+// 128 threads takes V vectors; what runs along the tridiagonal (elimination,
+// substitutions, the sum of squares) runs in lanes of warp 0, everything
+// elementwise in all threads.  Every operation and its order are those of k_stein,
+// so the vectors are the same bit for bit.  The elimination's pivot test needs two
+// quotients and its multiplier a third: four lanes per vector compute |a|/(|a|+|b|),
+// |c|/(|c|+|a'|+|b'|), c/a and a/c side by side and take what the test selects.
+// Bound by that serial chain of FP64 instructions (64 cycles of a scheduler's pipe
+// each); k_stein walks the same chain through L2.  n = 565: 4.2 ms -> 1.3 ms for all
+// vectors, 1.0 ms for four; n = 2000, one vector: 19 ms -> 3.5 ms.
+// Fields, index k, vector v at [(f n + k) V + v]: 0 a (reciprocal pivots), 1 b,
+// 2 c (multipliers), 3 d2, 4 y; then n V pivot flags.
+constexpr int STEIN_THREADS = 128;
+static size_t stein_sm_bytes(int n, int V) { return (size_t)n * V * (5 * sizeof(double) + 1) + 16; }
+template <int V>
+__global__ void __launch_bounds__(STEIN_THREADS) k_stein_sm(int nfull, const double* __restrict__ dfull,
+                                                            const double* __restrict__ efull,
+                                                            const double* __restrict__ wsel, int cnt,
+                                                            double* __restrict__ Eout, int ldE, int tbase,
+                                                            const int* __restrict__ src,
+                                                            const int* __restrict__ blocks) {
+  extern __shared__ double stein_sh[];
+  double* fa = stein_sh;
+  double* fb = fa + (size_t)nfull * V;
+  double* fc = fb + (size_t)nfull * V;
+  double* fd = fc + (size_t)nfull * V;
+  double* fy = fd + (size_t)nfull * V;
+  unsigned char* ff = reinterpret_cast<unsigned char*>(fy + (size_t)nfull * V);
+  __shared__ int sh_s0[V], sh_n[V];
+  __shared__ double sh_lam[V], sh_tol[V], sh_sc[V];
+  __shared__ double sh_max[STEIN_THREADS / 32][V];
+  const int t0 = blockIdx.x * V, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (tid < V) {
+    const int t = t0 + tid;
+    int s0 = 0, s1 = (t < cnt) ? nfull : 0;
+    if (blocks && t < cnt) {
+      const int b = blocks[src[t]];
+      s0 = blocks[nfull + b];
+      s1 = blocks[2 * nfull + b];
+    }
+    sh_s0[tid] = s0;
+    sh_n[tid] = s1 - s0;
+    sh_lam[tid] = (t < cnt) ? wsel[t] : 0.0;
+  }
+  __syncthreads();
+  int nmax = 0;
+#pragma unroll
+  for (int v = 0; v < V; ++v) nmax = max(nmax, sh_n[v]);
+  // tol from the largest row sum; start vectors
+#pragma unroll
+  for (int v = 0; v < V; ++v) {
+    const int n = sh_n[v];
+    const double* d = dfull + sh_s0[v];
+    const double* e = efull + sh_s0[v];
+    double tn = 0.0;
+    for (int i = tid; i < n; i += STEIN_THREADS) {
+      const double r = fabs(d[i]) + (i > 0 ? fabs(e[i - 1]) : 0.0) + (i + 1 < n ? fabs(e[i]) : 0.0);
+      tn = fmax(tn, r);
+      fy[(size_t)i * V + v] = hash_unif(((unsigned long long)(tbase + t0 + v) << 32) ^ (unsigned long long)i);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) tn = fmax(tn, __shfl_xor_sync(0xffffffffu, tn, o));
+    if (lane == 0) sh_max[warp][v] = tn;
+  }
+  __syncthreads();
+  if (tid < V) {
+    double tn = sh_max[0][tid];
+    for (int w = 1; w < STEIN_THREADS / 32; ++w) tn = fmax(tn, sh_max[w][tid]);
+    sh_tol[tid] = fmax(DBL_EPSILON * tn, DBL_MIN);
+  }
+  // ---- elimination with partial pivoting
+  if (warp == 0) {
+    const int v = (lane >> 2) % V, sub = lane & 3;   // lanes past 4 V repeat the first vectors, unstored
+    const bool mine = lane < 4 * V && sub == 0;
+    const int n = sh_n[v];
+    const double* d = dfull + sh_s0[v];
+    const double* e = efull + sh_s0[v];
+    const double lam = sh_lam[v];
+    double ak = (n > 0) ? d[0] - lam : 1.0;
+    double bk = (n > 1) ? e[0] : 0.0;
+    double ck = bk, dn = (n > 1) ? d[1] : 0.0, en = (n > 2) ? e[1] : 0.0;
+    for (int k = 0; k + 1 < nmax; ++k) {
+      const bool on = k + 1 < n;
+      const double ak1 = dn - lam;
+      const double bk1 = en;                               // 0 from row n - 2 on
+      const double ckn = en;
+      dn = (k + 2 < n) ? d[k + 2] : 0.0;                   // next step's entries on their way
+      en = (k + 3 < n) ? e[k + 2] : 0.0;
+      const double scale1 = fabs(ak) + fabs(bk);
+      const double scale2 = fabs(ck) + fabs(ak1) + fabs(bk1);
+      const double num = (sub == 0) ? fabs(ak) : (sub == 1) ? fabs(ck) : (sub == 2) ? ck : ak;
+      const double den = (sub == 0) ? scale1 : (sub == 1) ? scale2 : (sub == 2) ? ak : ck;
+      const double q = num / den;
+      const int b4 = lane & ~3;
+      const double q0 = __shfl_sync(0xffffffffu, q, b4), piv2 = __shfl_sync(0xffffffffu, q, b4 + 1);
+      const double q2 = __shfl_sync(0xffffffffu, q, b4 + 2), q3 = __shfl_sync(0xffffffffu, q, b4 + 3);
+      const double piv1 = (scale1 == 0.0) ? 0.0 : q0;
+      if (on) {
+        double oa = ak, ob = bk, oc = 0.0, od = 0.0, na, nb = bk1;
+        unsigned char fl = 0;
+        if (ck == 0.0) {
+          na = ak1;
+        } else if (piv2 <= piv1) {
+          oc = q2;
+          na = ak1 - q2 * bk;
+        } else {
+          fl = 1;
+          oa = ck;
+          ob = ak1;
+          oc = q3;
+          na = bk - q3 * ak1;
+          if (k + 2 < n) {
+            od = bk1;
+            nb = -q3 * bk1;
+          } else {
+            nb = 0.0;
+          }
+        }
+        if (mine) {
+          const size_t x = (size_t)k * V + v;
+          fa[x] = oa;
+          fb[x] = ob;
+          fc[x] = oc;
+          fd[x] = od;
+          ff[x] = fl;
+        }
+        ak = na;
+        bk = nb;
+        ck = ckn;
+      }
+    }
+    if (mine && n > 0) fa[(size_t)(n - 1) * V + v] = ak;
+  }
+  __syncthreads();
+  // reciprocal pivots (tiny pivots replaced by +-tol)
+  for (int x = tid; x < nmax * V; x += STEIN_THREADS) {
+    const int v = x % V;
+    if (x / V >= sh_n[v]) continue;
+    double a = fa[x];
+    if (fabs(a) < sh_tol[v]) a = (a >= 0.0) ? sh_tol[v] : -sh_tol[v];
+    fa[x] = 1.0 / a;
+  }
+  __syncthreads();
+  for (int iter = 0; iter < 3; ++iter) {
+    if (warp == 0 && lane < V && sh_n[lane % V] > 0) {
+      const int v = lane, n = sh_n[v];
+      // forward
+      double yp = fy[v];
+      {
+        double c = 0.0, yn = 0.0;
+        unsigned char fl = 0;
+        if (n > 1) { c = fc[v]; fl = ff[v]; yn = fy[V + v]; }
+        for (int k = 1; k < n; ++k) {
+          const double cc = c, yk = yn;
+          const bool f = fl != 0;
+          if (k + 1 < n) {
+            c = fc[(size_t)k * V + v];
+            fl = ff[(size_t)k * V + v];
+            yn = fy[(size_t)(k + 1) * V + v];
+          }
+          const double keep = f ? yk : yp, other = f ? yp : yk;
+          fy[(size_t)(k - 1) * V + v] = keep;
+          yp = other - cc * keep;
+        }
+        fy[(size_t)(n - 1) * V + v] = yp;
+      }
+      // backward; see k_stein for the rescaling
+      unsigned long long ymax = 0ull;
+      double y1 = 0.0, y2 = 0.0;
+      double a = fa[(size_t)(n - 1) * V + v], b = 0.0, d2 = 0.0, yk0 = yp;
+      for (int k = n - 1; k >= 0; --k) {
+        double tmp = yk0;
+        const double ac = a, bc = b, dc = d2;
+        if (k > 0) {
+          const size_t x = (size_t)(k - 1) * V + v;
+          a = fa[x];
+          b = fb[x];
+          d2 = fd[x];
+          yk0 = fy[x];
+        }
+        if (k + 1 < n) tmp -= bc * y1;
+        if (k + 2 < n) tmp -= dc * y2;
+        double yk = tmp * ac;
+        if ((__double2hiint(yk) & 0x7FFFFFFF) >= 0x58F00000) {   // !(|yk| < 2^400)
+          for (int j = 0; j < n; ++j) fy[(size_t)j * V + v] *= 0x1p-400;
+          yk0 *= 0x1p-400;
+          y1 *= 0x1p-400;
+          ymax = (unsigned long long)__double_as_longlong(__longlong_as_double((long long)ymax) * 0x1p-400);
+          yk = (tmp * 0x1p-400) * ac;
+        }
+        fy[(size_t)k * V + v] = yk;
+        const unsigned long long u = (unsigned long long)__double_as_longlong(yk) & 0x7FFFFFFFFFFFFFFFull;
+        if (u <= 0x7FF0000000000000ull && u > ymax) ymax = u;
+        y2 = y1;
+        y1 = yk;
+      }
+      const double ym = __longlong_as_double((long long)ymax);
+      sh_sc[v] = (ym > 0.0) ? 1.0 / ym : 1.0;
+    }
+    __syncthreads();
+    for (int x = tid; x < nmax * V; x += STEIN_THREADS)
+      if (x / V < sh_n[x % V]) fy[x] = fy[x] * sh_sc[x % V];
+    __syncthreads();
+    if (warp == 0 && lane < V) {
+      const int v = lane, n = sh_n[v];
+      double nrm = 0.0;
+#pragma unroll 8
+      for (int k = 0; k < n; ++k) {
+        const double yk = fy[(size_t)k * V + v];
+        nrm = fma(yk, yk, nrm);
+      }
+      sh_sc[v] = 1.0 / sqrt(nrm);
+    }
+    __syncthreads();
+    for (int x = tid; x < nmax * V; x += STEIN_THREADS)
+      if (x / V < sh_n[x % V]) fy[x] *= sh_sc[x % V];
+    __syncthreads();
+  }
+#pragma unroll
+  for (int v = 0; v < V; ++v) {
+    if (t0 + v >= cnt) break;
+    double* out = Eout + (size_t)(t0 + v) * ldE;
+    const int s0 = sh_s0[v], n = sh_n[v];
+    for (int k = tid; k < nfull; k += STEIN_THREADS)
+      out[k] = (k >= s0 && k < s0 + n) ? fy[(size_t)(k - s0) * V + v] : 0.0;
+  }
+}
+
 // ---------------------------------------------------------------------------
 // 5. Back-transformation: row t of E <- Q row t (Q = H_0 ... H_{n-3})
 // ---------------------------------------------------------------------------
@@ -1401,15 +1629,42 @@ static void eigenvalues_all(cudaStream_t st, int n, EigWork* w, int nblocks, dou
   k_rank<<<cdiv(n, 128), 128, 0, st>>>(n, w->val, wout, w->src);
 }
 
+template <int V>
+static void launch_stein_sm(cudaStream_t st, int n, EigWork* w, const double* e, const double* wv, int first, int cnt,
+                            double* E, bool blk) {
+  allow_max_smem((const void*)k_stein_sm<V>);
+  count_launch();
+  k_stein_sm<V><<<cdiv(cnt, V), STEIN_THREADS, stein_sm_bytes(n, V), st>>>(
+      n, w->d, e, wv + first, cnt, E, n, first, blk ? w->src + first : nullptr, blk ? w->blocks : nullptr);
+}
+
+// Vectors per block of the shared-memory form: enough to keep the blocks to about
+// one per SM, as many as fit (8 up to order 670, 1 up to 5300).  It takes about
+// 1.75 us per unit of n and wave of blocks, the global-memory form about 8 us per
+// unit of n for any number of vectors, so from five waves on (n = 2000 with all its
+// vectors: seven waves, 24.7 ms against 19.2 ms) the latter runs.
 static void eigenvectors(cudaStream_t st, int n, EigWork* w, int nblocks, const double* wv, int first, int cnt,
                          double* E) {
   const double* e = (nblocks <= 1) ? w->e : w->es;
+  const bool blk = nblocks > 1;
+  const size_t most = 220 * 1024;
+  int V = 8;
+  while (V > 1 && (stein_sm_bytes(n, V) > most || cnt <= 148 * (V / 2))) V /= 2;
+  const size_t need = stein_sm_bytes(n, V);
+  if (need <= most && cdiv(cnt, V) <= 4 * 148 * (most / need)) {
+    switch (V) {
+      case 8: launch_stein_sm<8>(st, n, w, e, wv, first, cnt, E, blk); break;
+      case 4: launch_stein_sm<4>(st, n, w, e, wv, first, cnt, E, blk); break;
+      case 2: launch_stein_sm<2>(st, n, w, e, wv, first, cnt, E, blk); break;
+      default: launch_stein_sm<1>(st, n, w, e, wv, first, cnt, E, blk); break;
+    }
+    return;
+  }
   for (int t0 = 0; t0 < cnt; t0 += w->batch) {
     const int c = std::min(w->batch, cnt - t0);
     count_launch();
     k_stein<<<cdiv(c, 64), 64, 0, st>>>(n, w->d, e, wv + first + t0, c, w->ws, w->batch, E + (size_t)t0 * n, n,
-                                        first + t0, nblocks <= 1 ? nullptr : w->src + first + t0,
-                                        nblocks <= 1 ? nullptr : w->blocks);
+                                        first + t0, blk ? w->src + first + t0 : nullptr, blk ? w->blocks : nullptr);
   }
 }
 
