@@ -1389,6 +1389,81 @@ __global__ void k_ormtr_rows(int n, const double* __restrict__ A, int lda, const
   }
 }
 
+// The same with the vectors and the reflectors in shared memory: a warp per vector,
+// the warps of a block share the reflector of a step, which cp.async fetches two
+// steps ahead.  Same lanes, same sums, same result.  Bound by the FP64 pipe where
+// several warps share an SM, by a step's chain (the lane's multiply-adds, the warp
+// sum) where they do not; k_ormtr_rows waits for L2 twice a step.
+constexpr int ORM_STAGES = 3;
+static size_t ormtr_sm_bytes(int n, int warps) { return (size_t)(warps + ORM_STAGES + 1) * n * sizeof(double); }
+__global__ void __launch_bounds__(256) k_ormtr_sm(int n, const double* __restrict__ A, int lda,
+                                                  const double* __restrict__ tauh, double* __restrict__ E, int ldE,
+                                                  int rows) {
+  extern __shared__ double orm_sh[];
+  const int nw = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double* x = orm_sh + (size_t)warp * n;
+  double* ring = orm_sh + (size_t)nw * n;
+  double* st = ring + (size_t)ORM_STAGES * n;
+  const int t = blockIdx.x * nw + warp;
+  const bool have = t < rows;
+  for (int l = lane; l < n; l += 32) x[l] = have ? E[(size_t)t * ldE + l] : 0.0;
+  for (int l = threadIdx.x; l < n; l += blockDim.x) st[l] = tauh[l];
+  auto fetch = [&](int j, int slot) {
+    if (j >= 0) {
+      const double* src = A + (size_t)j * lda + j + 1;
+      double* dst = ring + (size_t)slot * n;
+      for (int l = threadIdx.x; l < n - j - 1; l += blockDim.x)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(
+                         static_cast<uint32_t>(__cvta_generic_to_shared(dst + l))),
+                     "l"(src + l)
+                     : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  fetch(n - 3, 0);
+  fetch(n - 4, 1);
+  int slot = 0;
+  for (int j = n - 3; j >= 0; --j) {
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncthreads();   // reflector j is there for every warp, and slot + 2 has been read
+    fetch(j - 2, slot >= 1 ? slot - 1 : slot + 2);
+    const double tau = st[j];
+    if (tau != 0.0) {
+      const double* vj = ring + (size_t)slot * n;
+      double* xj = x + j + 1;
+      const int len = n - j - 1;
+      double s = 0.0;
+#pragma unroll 4
+      for (int l = lane; l < len; l += 32) s = fma(vj[l], xj[l], s);
+      s = wsum(s) * tau;
+#pragma unroll 4
+      for (int l = lane; l < len; l += 32) xj[l] -= s * vj[l];
+      __syncwarp();
+    }
+    slot = (slot == ORM_STAGES - 1) ? 0 : slot + 1;
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  if (have)
+    for (int l = lane; l < n; l += 32) E[(size_t)t * ldE + l] = x[l];
+}
+// Warps per block: about one block per SM; from 592 vectors on eight, so that every
+// scheduler has a second warp to issue while one waits.  Orders whose working set
+// does not fit (above 2300 with eight warps, 3500 with four) run k_ormtr_rows.
+// All vectors and the top ones of a build together: n = 565 4.0 -> 1.8 ms, n = 2000
+// 47 -> 28 ms.
+static void ormtr(cudaStream_t st, int n, const double* A, int lda, const double* tauh, double* E, int ldE, int rows) {
+  count_launch();
+  int nw = (rows > 4 * 148) ? 8 : (rows > 2 * 148) ? 4 : (rows > 148) ? 2 : 1;
+  if (nw == 8 && ormtr_sm_bytes(n, nw) > 220 * 1024) nw = 4;
+  const size_t smem = ormtr_sm_bytes(n, nw);
+  if (smem <= 220 * 1024) {
+    allow_max_smem((const void*)k_ormtr_sm);
+    k_ormtr_sm<<<cdiv(rows, nw), 32 * nw, smem, st>>>(n, A, lda, tauh, E, ldE, rows);
+    return;
+  }
+  k_ormtr_rows<<<cdiv((size_t)rows * 32, 256), 256, 0, st>>>(n, A, lda, tauh, E, ldE, rows);
+}
+
 // Modified Gram-Schmidt over `rows` (<= 32) vectors of length n, one CTA.
 __global__ void k_mgs(int n, double* E, int ldE, int rows) {
   __shared__ double red[32];
@@ -1710,8 +1785,7 @@ sdp_status eig_full(cudaStream_t st, int n, double* A, double* wout, double* E, 
     potrf(st, n, w->G, n, w->info, w->aux);
     trsm_left_lower(st, false, n, n, w->G, n, E, n, w->aux);
   }
-  count_launch();
-  k_ormtr_rows<<<cdiv((size_t)n * 32, 256), 256, 0, st>>>(n, A, n, w->tauh, E, n, n);
+  ormtr(st, n, A, n, w->tauh, E, n, n);
   return SDP_OK;
 }
 
@@ -1742,8 +1816,8 @@ sdp_status eig_extremes(cudaStream_t st, int n, double* A, int k, double* lmin_d
     SDP_CK_ST(cudaMemcpyAsync(wtop, w->wsel + n - k, k * sizeof(double), cudaMemcpyDeviceToDevice, st));
     eigenvectors(st, n, w, nb, w->wsel, n - k, k, Etop);
   }
-  count_launch(2);
-  k_ormtr_rows<<<cdiv((size_t)k * 32, 128), 128, 0, st>>>(n, A, n, w->tauh, Etop, n, k);
+  ormtr(st, n, A, n, w->tauh, Etop, n, k);
+  count_launch();
   k_mgs<<<1, 256, 0, st>>>(n, Etop, n, k);
   return SDP_OK;
 }
