@@ -68,42 +68,55 @@ __device__ __forceinline__ double lz_start(int i) {
   return (double)(z >> 11) * 0x1p-52 - 1.0;
 }
 
-// Sturm count of T (diagonal a[0..j), off-diagonal b[0..j-1)) below x
-__device__ int lz_sturm(int j, const double* a, const double* b, double x) {
+// Sturm count of T (diagonal a[0..j), nb[i] = -b_i^2 rounded) below x.  Signs, the
+// zero test and the range test look at the bits: an FP64 compare would hold the
+// pipe as long as a multiply-add.
+__device__ int lz_sturm(int j, const double* a, const double* nb, double x) {
+  const unsigned long long mag = 0x7FFFFFFFFFFFFFFFull;
   double pm = 1.0, p = a[0] - x;
-  int sp = (p > 0.0) ? 1 : -1;
-  int cnt = (sp < 0) ? 1 : 0;
+  bool neg = !(p > 0.0);
+  int cnt = neg ? 1 : 0;
   for (int i = 1; i < j; ++i) {
-    const double pn = fma(a[i] - x, p, -b[i - 1] * b[i - 1] * pm);
-    const int sn = (pn > 0.0) ? 1 : (pn < 0.0 ? -1 : -sp);
-    cnt += (sn != sp);
-    sp = sn;
+    const double pn = fma(a[i] - x, p, nb[i - 1] * pm);
+    const unsigned long long un = (unsigned long long)__double_as_longlong(pn) & mag;
+    const bool sn = (un - 1ull >= 0x7FF0000000000000ull) ? !neg : __double2hiint(pn) < 0;   // zero or NaN: a change
+    cnt += (sn != neg) ? 1 : 0;
+    neg = sn;
+    const unsigned long long up = (unsigned long long)__double_as_longlong(p) & mag;
     pm = p;
     p = pn;
-    const double m = fmax(fabs(p), fabs(pm));
-    if (m > 0x1p+400) { p *= 0x1p-400; pm *= 0x1p-400; }
-    else if (m < 0x1p-400 && m > 0.0) { p *= 0x1p+400; pm *= 0x1p+400; }
+    const unsigned long long um = un > up ? un : up;
+    if (um > 0x58F0000000000000ull) { p *= 0x1p-400; pm *= 0x1p-400; }                      // above 2^400
+    else if (um < 0x26F0000000000000ull && um > 0ull) { p *= 0x1p+400; pm *= 0x1p+400; }    // below 2^-400
   }
   return cnt;
 }
 
 // One warp: theta = lambda_min(T_j) by 32-way multisection, then the last
 // entry of its unit eigenvector by two steps of inverse iteration (lane 0).
-// res[0] = theta, res[1] = |s_last|.
+// res[0] = theta, res[1] = |s_last|.  work: 6 LZ_MAXIT doubles.
 __device__ void lz_ritz_min(int j, const double* a, const double* b, double* res, double* work) {
   const int lane = threadIdx.x & 31;
   double lo = a[0], hi = a[0];
-  for (int i = 0; i < j; ++i) {
+  for (int i = lane; i < j; i += 32) {
     const double r = (i > 0 ? fabs(b[i - 1]) : 0.0) + (i + 1 < j ? fabs(b[i]) : 0.0);
     lo = fmin(lo, a[i] - r);
     hi = fmax(hi, a[i] + r);
   }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+    hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+  }
+  double* nb = work + 5 * LZ_MAXIT;   // -b_i^2
+  for (int i = lane; i + 1 < j; i += 32) nb[i] = -b[i] * b[i];
+  __syncwarp();
   const double pad = 4.0 * DBL_EPSILON * fmax(fabs(lo), fabs(hi)) * j + DBL_MIN;
   lo -= pad;
   hi += pad;
   for (int it = 0; it < 14; ++it) {
     const double x = lo + (hi - lo) * (double)(lane + 1) / 33.0;
-    const int c = lz_sturm(j, a, b, x);
+    const int c = lz_sturm(j, a, nb, x);
     const unsigned ge = __ballot_sync(0xffffffffu, c >= 1);
     if (ge == 0u) {
       lo = lo + (hi - lo) * 32.0 / 33.0;
@@ -119,39 +132,56 @@ __device__ void lz_ritz_min(int j, const double* a, const double* b, double* res
   if (lane == 0) {
     const double theta = 0.5 * (lo + hi);
     // inverse iteration: (T - theta I) s = s_prev, Gaussian elimination with
-    // partial pivoting on the tridiagonal (work: 4 j doubles)
+    // partial pivoting on the tridiagonal; the first pass keeps the multipliers
+    // and interchanges, the second applies them
     double* s = work;
-    double* dd = work + j;       // diagonal after elimination
-    double* du = work + 2 * j;   // first superdiagonal
-    double* du2 = work + 3 * j;  // second superdiagonal (from pivoting)
+    double* dd = work + LZ_MAXIT;       // diagonal after elimination
+    double* du = work + 2 * LZ_MAXIT;   // first superdiagonal
+    double* du2 = work + 3 * LZ_MAXIT;  // second superdiagonal (from pivoting)
+    double* ll = work + 4 * LZ_MAXIT;   // multipliers
+    unsigned long long sw0 = 0ull, sw1 = 0ull;   // rows interchanged at step i (LZ_MAXIT <= 128)
     const double tiny = fmax(fabs(theta), 1.0) * 1e-300 + DBL_MIN;
     for (int i = 0; i < j; ++i) s[i] = 1.0;
     for (int rep = 0; rep < 2; ++rep) {
-      // factor rows in place into upper band (dd, du, du2), apply to s
-      double cd = a[0] - theta, cu = (j > 1) ? b[0] : 0.0;
-      for (int i = 0; i < j; ++i) {
-        if (i + 1 < j) {
-          const double sub = b[i];
-          const double nd = a[i + 1] - theta;
-          const double nu = (i + 2 < j) ? b[i + 1] : 0.0;
-          if (fabs(cd) >= fabs(sub)) {
-            const double piv = (cd != 0.0) ? cd : tiny;
-            const double l = sub / piv;
-            dd[i] = piv; du[i] = cu; du2[i] = 0.0;
-            s[i + 1] -= l * s[i];
-            cd = nd - l * cu;
-            cu = nu;
+      if (rep == 0) {
+        // factor rows in place into upper band (dd, du, du2), apply to s
+        double cd = a[0] - theta, cu = (j > 1) ? b[0] : 0.0;
+        for (int i = 0; i < j; ++i) {
+          if (i + 1 < j) {
+            const double sub = b[i];
+            const double nd = a[i + 1] - theta;
+            const double nu = (i + 2 < j) ? b[i + 1] : 0.0;
+            if (fabs(cd) >= fabs(sub)) {
+              const double piv = (cd != 0.0) ? cd : tiny;
+              const double l = sub / piv;
+              ll[i] = l;
+              dd[i] = piv; du[i] = cu; du2[i] = 0.0;
+              s[i + 1] -= l * s[i];
+              cd = nd - l * cu;
+              cu = nu;
+            } else {
+              const double l = cd / sub;
+              ll[i] = l;
+              if (i < 64) sw0 |= 1ull << i;
+              else sw1 |= 1ull << (i - 64);
+              dd[i] = sub; du[i] = nd; du2[i] = nu;
+              const double t = s[i];
+              s[i] = s[i + 1];
+              s[i + 1] = t - l * s[i];
+              cd = cu - l * nd;
+              cu = -l * nu;
+            }
           } else {
-            const double l = cd / sub;
-            dd[i] = sub; du[i] = nd; du2[i] = nu;
-            const double t = s[i];
-            s[i] = s[i + 1];
-            s[i + 1] = t - l * s[i];
-            cd = cu - l * nd;
-            cu = -l * nu;
+            dd[i] = (cd != 0.0) ? cd : tiny;
           }
-        } else {
-          dd[i] = (cd != 0.0) ? cd : tiny;
+        }
+      } else {
+        for (int i = 0; i + 1 < j; ++i) {
+          const bool swp = ((i < 64 ? sw0 >> i : sw1 >> (i - 64)) & 1ull) != 0ull;
+          const double l = ll[i], s0 = s[i], s1 = s[i + 1];
+          const double keep = swp ? s1 : s0, other = swp ? s0 : s1;
+          s[i] = keep;
+          s[i + 1] = other - l * keep;
         }
       }
       for (int i = j - 1; i >= 0; --i) {
@@ -208,7 +238,7 @@ __global__ void __cluster_dims__(LZ_CS, 1, 1) __launch_bounds__(LZ_THREADS)
   double* t1 = sm + 4 * (size_t)n;  // n   A3 q   (three-factor operator)
   double* t2 = sm + 5 * (size_t)n;  // n   A2 A3 q
   __shared__ double alpha[LZ_MAXIT], beta[LZ_MAXIT], cdot[LZ_MAXIT + 1];
-  __shared__ double red[32], ritz[2], twork[4 * LZ_MAXIT];
+  __shared__ double red[32], ritz[2], twork[6 * LZ_MAXIT];
   __shared__ int stop;
   const int rank = (int)cluster.block_rank();
   double* Q = Qall + (size_t)rank * (LZ_MAXIT + 1) * n;
@@ -314,6 +344,247 @@ __global__ void __cluster_dims__(LZ_CS, 1, 1) __launch_bounds__(LZ_THREADS)
   cluster.sync();   // no CTA leaves while another may still write into its shared memory
 }
 
+// ---------------------------------------------------------------------------
+// The same iteration over the whole GPU (cooperative launch), for orders where 8
+// SMs' FP64 pipes bound the three products.  Every sum keeps its order -- a
+// row of a product, a reorthogonalisation coefficient and an entry's correction
+// are one warp's or one thread's work in either form, the block sums are formed by
+// 256 threads in every CTA -- so both forms return the same bits.  Work is dealt
+// over all warps and meets in global memory after a grid barrier: three products,
+// then per Gram-Schmidt pass the coefficients and the corrected vector (seven
+// barriers a step).  For A1 A2 A3 with A1 lower and A3 upper triangular the
+// stored zeros are skipped.  The convergence test is a serial computation of tens
+// of microseconds, so an extra CTA runs it while the others go on; when it says
+// stop, the (at most six) steps done meanwhile are dropped.  Every wait is
+// bounded; one that runs out ends the kernel with "not converged".
+// ---------------------------------------------------------------------------
+constexpr long long LZ_SPIN_CYCLES = 4000000000ll;
+constexpr int LZ_CHECKS = LZ_MAXIT / LZ_CHECK + 2;
+struct LzCtl {                 // zeroed before the launch
+  unsigned int arrived;        // grid barrier: arrivals so far
+  int fail;                    // a wait ran out
+  int stop;                    // the test has accepted an estimate
+  int halt;                    // workers leave at this step (0: go on), set by CTA 0
+  int req[LZ_CHECKS];          // requested tests: steps, + 1024 for an invariant subspace
+};
+__device__ __forceinline__ int lz_ld(const int* p) {
+  int v;
+  asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void lz_st(int* p, int v) {
+  asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+// All workers arrive; false when the wait ran out somewhere.
+__device__ bool lz_barrier(LzCtl* c, unsigned int target) {
+  __shared__ int s_ok;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(&c->arrived, 1u);
+    const long long t0 = clock64();
+    int ok = 1;
+    while ((unsigned int)lz_ld(reinterpret_cast<const int*>(&c->arrived)) < target) {
+      if (lz_ld(&c->fail)) { ok = 0; break; }
+      if (clock64() - t0 > LZ_SPIN_CYCLES) { lz_st(&c->fail, 1); ok = 0; break; }
+    }
+    __threadfence();
+    s_ok = ok;
+  }
+  __syncthreads();
+  return s_ok != 0;
+}
+
+// y[r] = A[r, :] x, rows dealt over the warps of all workers; shape 0 full, 1 lower, 2 upper
+__device__ __forceinline__ void lz_gemv(int n, const double* __restrict__ A, int lda, const double* x, double* y,
+                                        int gw, int nwarps, int lane, int shape) {
+  for (int r = gw; r < n; r += nwarps) {
+    const double* ar = A + (size_t)r * lda;
+    const int c0 = (shape == 2) ? (r & ~31) : 0, c1 = (shape == 1) ? min(n, (r & ~31) + 32) : n;
+    double acc = 0.0;
+#pragma unroll 8
+    for (int c = c0 + lane; c < c1; c += 32) acc = fma(ar[c], x[c], acc);
+    acc = lz_warp_sum(acc);
+    if (lane == 0) __stcg(y + r, acc);
+  }
+}
+
+__global__ void __launch_bounds__(LZ_THREADS)
+    k_lanczos_grid(int n, const double* __restrict__ M, const double* __restrict__ A2, const double* __restrict__ A3,
+                   int ldm, double rtol, double accept_above, double* __restrict__ buf, double* __restrict__ out,
+                   LzCtl* ctl) {
+  extern __shared__ double sm[];
+  double* q = sm;                   // n   current q
+  double* wb = sm + n;              // n   product, then the next direction
+  double* qp = sm + 2 * (size_t)n;  // n   previous q
+  double* tv = sm + 3 * (size_t)n;  // n   A3 q, A2 A3 q
+  __shared__ double red[32], cdot[LZ_MAXIT + 1];
+  double* Q = buf;                                     // (LZ_MAXIT + 1) x n
+  double* g1 = buf + (size_t)(LZ_MAXIT + 1) * n;       // n each: exchanged vectors
+  double* g2 = g1 + n;
+  double* g3 = g2 + n;
+  double* gc = g3 + n;                                 // 2 x (LZ_MAXIT + 1): coefficients of the two passes
+  double* ga = gc + 2 * (LZ_MAXIT + 1);                // alpha, beta
+  double* gb = ga + LZ_MAXIT;
+  const int G = (int)gridDim.x - 1;                    // workers; the last CTA tests
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int maxit = min(LZ_MAXIT, n);
+
+  if ((int)blockIdx.x == G) {
+    __shared__ double alpha[LZ_MAXIT], beta[LZ_MAXIT], ritz[2], twork[6 * LZ_MAXIT];
+    __shared__ int s_req;
+    for (int ci = 0; ci < LZ_CHECKS; ++ci) {
+      if (threadIdx.x == 0) {
+        const long long t0 = clock64();
+        int rq;
+        while ((rq = lz_ld(&ctl->req[ci])) == 0) {
+          if (lz_ld(&ctl->fail)) break;
+          if (clock64() - t0 > LZ_SPIN_CYCLES) { lz_st(&ctl->fail, 1); break; }
+        }
+        s_req = rq;
+      }
+      __syncthreads();
+      const int rq = s_req;
+      if (rq == 0) {
+        if (threadIdx.x == 0) out[4] = 0.0;
+        return;
+      }
+      const int steps = rq & 1023;
+      const bool invariant = rq >= 1024;
+      for (int i = threadIdx.x; i < steps; i += blockDim.x) {
+        alpha[i] = __ldcg(ga + i);
+        beta[i] = __ldcg(gb + i);
+      }
+      __syncthreads();
+      if (warp == 0) lz_ritz_min(steps, alpha, beta, ritz, twork);
+      __syncthreads();
+      const double theta = ritz[0], bound = invariant ? 0.0 : beta[steps - 1] * ritz[1];
+      const bool ok = invariant || bound <= rtol * fabs(theta) ||
+                      (steps >= 2 * LZ_CHECK && theta - bound >= accept_above);
+      if (ok || steps == maxit) {
+        if (threadIdx.x == 0) {
+          out[0] = theta - bound;
+          out[1] = theta;
+          out[2] = bound;
+          out[3] = (double)steps;
+          out[4] = ok ? 1.0 : 0.0;
+          lz_st(&ctl->stop, 1);
+        }
+        return;
+      }
+      __syncthreads();
+    }
+    return;
+  }
+
+  const int gw = (int)blockIdx.x * (LZ_THREADS / 32) + warp, nwarps = G * (LZ_THREADS / 32);
+  const int gt = (int)blockIdx.x * LZ_THREADS + (int)threadIdx.x, nthr = G * LZ_THREADS;
+  unsigned int target = 0;
+  auto sync = [&]() {
+    target += (unsigned)G;
+    return lz_barrier(ctl, target);
+  };
+  double s = 0.0;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    const double v = lz_start(i);
+    q[i] = v;
+    qp[i] = 0.0;
+    s = fma(v, v, s);
+  }
+  s = lz_block_sum(s, red);
+  const double inv0 = 1.0 / sqrt(s);
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    q[i] *= inv0;
+    if (blockIdx.x == 0) __stcg(Q + i, q[i]);
+  }
+  double bprev = 0.0;
+  int checks = 0;
+  __syncthreads();
+  for (int j = 0; j < maxit; ++j) {
+    if (A2) {
+      lz_gemv(n, A3, ldm, q, g1, gw, nwarps, lane, 2);
+      if (!sync()) return;
+      for (int i = threadIdx.x; i < n; i += blockDim.x) tv[i] = __ldcg(g1 + i);
+      __syncthreads();
+      lz_gemv(n, A2, ldm, tv, g2, gw, nwarps, lane, 0);
+      if (!sync()) return;
+      for (int i = threadIdx.x; i < n; i += blockDim.x) tv[i] = __ldcg(g2 + i);
+      __syncthreads();
+      lz_gemv(n, M, ldm, tv, g3, gw, nwarps, lane, 1);
+    } else {
+      lz_gemv(n, M, ldm, q, g3, gw, nwarps, lane, 0);
+    }
+    if (!sync()) return;
+    double a = 0.0;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+      wb[i] = __ldcg(g3 + i);
+      a = fma(q[i], wb[i], a);
+    }
+    a = lz_block_sum(a, red);
+    for (int i = threadIdx.x; i < n; i += blockDim.x) wb[i] = wb[i] - a * q[i] - bprev * qp[i];
+    __syncthreads();
+    for (int pass = 0; pass < 2; ++pass) {
+      double* cg_ = gc + pass * (LZ_MAXIT + 1);
+      double* gv = pass ? g2 : g1;
+      for (int t = gw; t <= j; t += nwarps) {
+        const double* qt = Q + (size_t)t * n;
+        double c = 0.0;
+#pragma unroll 8
+        for (int i = lane; i < n; i += 32) c = fma(__ldcg(qt + i), wb[i], c);
+        c = lz_warp_sum(c);
+        if (lane == 0) __stcg(cg_ + t, c);
+      }
+      if (!sync()) return;
+      for (int t = threadIdx.x; t <= j; t += blockDim.x) cdot[t] = __ldcg(cg_ + t);
+      __syncthreads();
+      for (int i = gt; i < n; i += nthr) {
+        double v = wb[i];
+#pragma unroll 8
+        for (int t = 0; t <= j; ++t) v = fma(-cdot[t], __ldcg(Q + (size_t)t * n + i), v);
+        __stcg(gv + i, v);
+      }
+      if (pass == 1 && blockIdx.x == 0 && threadIdx.x == 0 && lz_ld(&ctl->stop)) lz_st(&ctl->halt, j + 1);
+      if (!sync()) return;
+      for (int i = threadIdx.x; i < n; i += blockDim.x) wb[i] = __ldcg(gv + i);
+      __syncthreads();
+    }
+    double b2 = 0.0;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) b2 = fma(wb[i], wb[i], b2);
+    b2 = lz_block_sum(b2, red);
+    const double b = sqrt(b2);
+    const int steps = j + 1;
+    const bool invariant = !(b > 1e-14 * fmax(fabs(a), fabs(bprev)) + DBL_MIN);
+    const bool check = invariant || steps == maxit || (steps % LZ_CHECK) == 0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      __stcg(ga + j, a);
+      __stcg(gb + j, b);
+      if (check) {
+        __threadfence();
+        lz_st(&ctl->req[checks], steps + (invariant ? 1024 : 0));
+      }
+    }
+    checks += check ? 1 : 0;
+    if (invariant || steps == maxit) return;
+    const int halt = lz_ld(&ctl->halt);   // written before this step's last barrier, for this step or an earlier one
+    if (halt != 0 && halt <= steps) return;
+    const double ib = 1.0 / b;
+    double* qn = Q + (size_t)(j + 1) * n;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+      qp[i] = q[i];
+      const double v = wb[i] * ib;
+      q[i] = v;
+      if (blockIdx.x == 0) __stcg(qn + i, v);
+    }
+    bprev = b;
+    __syncthreads();
+  }
+}
+
+// Orders from which the whole-GPU form runs.
+constexpr int LZ_GRID_MIN_N = 256;
+
+// Basis copies of the cluster form, or one basis, the exchanged vectors and the
+// control block of the whole-GPU form.
 size_t lanczos_work_doubles(int n) { return (size_t)LZ_CS * (LZ_MAXIT + 1) * n + 8; }
 
 // Launch on st; results land in out_dev[0..4] (device).
@@ -325,6 +596,27 @@ sdp_status lanczos_min(cudaStream_t st, int n, const double* M, const double* A2
   const size_t smem = 6 * (size_t)n * sizeof(double);
   if (!lanczos_fits(n) || (A2 == nullptr) != (A3 == nullptr)) return SDP_ERR_UNSUPPORTED;
   allow_max_smem((const void*)k_lanczos_min);
+  if (n >= LZ_GRID_MIN_N) {
+    static int sms = 0;
+    if (!sms) {
+      int dev = 0;
+      cudaGetDevice(&dev);
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    }
+    // a warp per row, at most one CTA per SM, one SM for the test
+    const int G = std::min((n + LZ_THREADS / 32 - 1) / (LZ_THREADS / 32), sms - 1);
+    LzCtl* ctl = reinterpret_cast<LzCtl*>(work + lanczos_work_doubles(n) - (sizeof(LzCtl) + 7) / 8);
+    const size_t sg = 4 * (size_t)n * sizeof(double);
+    allow_max_smem((const void*)k_lanczos_grid);
+    if (cudaMemsetAsync(ctl, 0, sizeof(LzCtl), st) != cudaSuccess) return SDP_ERR_CUDA;
+    void* args[] = {&n, &M, &A2, &A3, &ldm, &rtol, &accept_above, &work, &out_dev, &ctl};
+    count_launch();
+    ktimer_begin(st, "lanczos");
+    const cudaError_t e = cudaLaunchCooperativeKernel((void*)k_lanczos_grid, dim3(G + 1), dim3(LZ_THREADS), args, sg, st);
+    ktimer_end(st, "lanczos", 0.0, 0.0);
+    if (e == cudaSuccess) return SDP_OK;
+    cudaGetLastError();   // no room for a cooperative grid: the cluster form
+  }
   count_launch();
   ktimer_begin(st, "lanczos");
   k_lanczos_min<<<LZ_CS, LZ_THREADS, smem, st>>>(n, M, A2, A3, ldm, rtol, accept_above, work, out_dev);

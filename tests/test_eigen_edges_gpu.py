@@ -94,3 +94,29 @@ def test_nt_scaling_at_edge_orders(n):
         prob.ipm_step()
         W = prob.get_W().cpu().numpy()
     assert np.linalg.norm(W @ S @ W - X) <= 50 * n * EPS * 16.0 * np.linalg.norm(X)
+
+
+@pytest.mark.parametrize("n", [63, 64, 255, 256, 257, 519, 1025, 2047])
+def test_step_length_is_close_to_the_boundary(n):
+    """alpha = min(1, 0.9 / -(theta - bound)) with bound <= 1e-3 |theta| and theta - bound <=
+    lambda_min(L^-1 dX L^-T) up to rounding: 0.998 of the largest step at least, never beyond it
+    (both sides of the order where the whole-GPU Lanczos takes over, and of the matrix sizes of
+    the resident tridiagonalisation)."""
+    d = si.unit_diag_instance(n)
+    rng = np.random.default_rng(n)
+    q = min(n, 8)   # spectra without an n x n factorisation: I + low rank
+    U, V = rng.standard_normal((n, q)) / np.sqrt(n), rng.standard_normal((n, q)) / np.sqrt(n)
+    X, S = 0.7 * np.eye(n) + U @ U.T, 0.9 * np.eye(n) + V @ V.T
+    with _prob(d) as prob:
+        prob.set_state(X, np.zeros(d.m), S, 0)
+        info = prob.ipm_step()
+        X1, _, _ = prob.get_solution()
+        W = prob.get_W().cpu().numpy()
+    assert np.linalg.norm(W @ S @ W - X) <= 50 * n * EPS * 16.0 * np.linalg.norm(X)
+    a = info["alpha_p"]
+    if a >= 1.0:
+        return
+    L = np.linalg.cholesky(X)
+    D = np.linalg.solve(L, np.linalg.solve(L, (X1 - X) / a).T)
+    amax = -1.0 / np.linalg.eigvalsh((D + D.T) / 2)[0]
+    assert 0.9 * 0.998 * amax * (1 - 1e-7) <= a <= 0.9 * amax * (1 + 1e-7)
