@@ -687,30 +687,34 @@ __global__ void __launch_bounds__(SY_THREADS) k_sytrd_cluster_smem(int n, double
 // With lower storage, p = A22 v splits into a row part (the owner's dot of its
 // lower row with v) and a column part (for column c, the sum over rows i > c
 // of A[i][c] v_i, which every CTA forms over its own rows).  Per column j:
-//   0: every CTA builds the reflector from the column j that the owners of
-//      rows i > j broadcast into vn at the end of column j - 1;
-//   1: row parts (warp per owned row) and the CTA's column parts (thread per
-//      column); cluster barrier;
+//   1: the CTA's column parts (thread per column) and row parts (warp per owned
+//      row); cluster barrier;
 //   2: the owner of row i adds its row part to the 16 CTAs' column parts for i
 //      (fixed order), scales by tau and broadcasts p_i and its share of p^T v;
 //      cluster barrier;
-//   3: w = p - (tau / 2)(p^T v) v; owned rows updated on c in [j + 1, i];
-//      the reflector is stored in column j of the owned rows, and column
-//      j + 1 is broadcast into vn; cluster barrier.
-// Remote buffers and the barriers that order them: vn is written in step 3
-// and read in step 0 of the next column (barrier 3 between; the next writes
-// come after barriers 1 and 2); part is read remotely between barriers 1 and
-// 2 and reused as w after barrier 2; p and kpart are written remotely
-// between barriers 1 and 2 and read after barrier 2.  Every sum runs in a
-// fixed order, so the result does not depend on timing.  At the end the
-// rows are written back with the lower part mirrored into the upper one:
-// row j then holds the reflector in A[j][j+1..], as the back-transformation
-// expects.
+//   3: w = p - (tau / 2)(p^T v) v.  Every CTA has column j + 1 as it was before this
+//      update (the owners broadcast it a column earlier) and updates it itself, so
+//      the next reflector starts at once: one warp forms its scalars while the
+//      warps of the other three schedulers update the owned rows on c in [j + 1, i],
+//      store the reflector in column j and broadcast column j + 2.
+// Three vectors rotate: b0 the reflector, b1 column j + 1, b2 first the column
+// parts, then column j + 2.  Remote writes and the barriers that order them: b2 is
+// written in step 3, after barrier 2 ended the reading of the column parts, and read
+// in step 3 of the next column; p and kpart are written between barriers 1 and 2
+// and read after barrier 2.  Every sum runs in a fixed order (those over the
+// reflector in 512 threads' order, p^T v in that of 16 warps), so the result does not
+// depend on timing.  An FP64 warp instruction holds its scheduler's pipe for 64
+// cycles: at n = 565 that bounds the first columns (14 us), latency the last ones.
+// With three barriers, 512 threads and the scalars on the way of the update a
+// column took 15.4 us on average (n = 565: 8.7 ms), now 12.0 us (6.8 ms).  At the end the rows are written back with
+// the lower part mirrored into the upper one: row j then holds the reflector in
+// A[j][j+1..], as the back-transformation expects.
+constexpr int SYL_THREADS = 1024;
 __device__ __forceinline__ size_t sy_off(int sl, int cs, int rank) {
   return (size_t)cs * sl * (sl - 1) / 2 + (size_t)sl * (rank + 1);
 }
-__global__ void __launch_bounds__(SY_THREADS) k_sytrd_cluster_lower(int n, double* A, int lda, double* d, double* e,
-                                                                     double* tauh) {
+__global__ void __launch_bounds__(SYL_THREADS, 1) k_sytrd_cluster_lower(int n, double* A, int lda, double* d,
+                                                                         double* e, double* tauh) {
   cg::cluster_group cluster = cg::this_cluster();
   const int cs = (int)cluster.num_blocks();
   const int rank = (int)cluster.block_rank();
@@ -719,56 +723,83 @@ __global__ void __launch_bounds__(SY_THREADS) k_sytrd_cluster_lower(int n, doubl
   // the vectors come first, at the same offset in every CTA (a remote access
   // maps the local offset); the packed rows, whose length depends on the
   // rank, follow them
-  double* v = sm;               // n: the reflector of the current column
-  double* vn = v + n;           // n: the next column (written remotely)
-  double* part = vn + n;        // n: column parts (read remotely), then w
-  double* p = part + n;         // n: tau A22 v (written remotely)
-  double* rowp = p + n;         // ceil(n / cs): row parts of the owned rows
+  double* p = sm + 3 * (size_t)n;   // n: tau A22 v (written remotely), then w
+  double* rowp = p + n;             // ceil(n / cs): row parts, then p_i, of the owned rows
   double* rows = rowp + (n + cs - 1) / cs;
   __shared__ double kpart[32];
   __shared__ double red[32];
-  __shared__ double s_tau, s_beta, s_scale;
-  const int wpb = blockDim.x / 32, wid = threadIdx.x / 32, lane = threadIdx.x % 32;
+  __shared__ double s_tau, s_beta, s_scale, s_K, s_w0;
+  const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31, nw = SYL_THREADS / 32;
   for (int sl = 0; sl < slots; ++sl) {
     const int i = sl * cs + rank;
     double* ri = rows + sy_off(sl, cs, rank);
-    for (int c = threadIdx.x; c <= i; c += blockDim.x) ri[c] = __ldcg(A + (size_t)i * lda + c);
+    for (int c = tid; c <= i; c += SYL_THREADS) ri[c] = __ldcg(A + (size_t)i * lda + c);
   }
   cluster.sync();
-  // column 0 into every CTA's vn
-  for (int sl = wid; sl < slots; sl += wpb) {
+  // columns 0 and 1 to every CTA
+  for (int sl = wid; sl < slots; sl += nw) {
     const int i = sl * cs + rank;
-    if (i >= 1 && lane < cs) cluster.map_shared_rank(vn, lane)[i - 1] = rows[sy_off(sl, cs, rank)];
+    const double* ri = rows + sy_off(sl, cs, rank);
+    if (i >= 1 && lane < cs) cluster.map_shared_rank(sm, lane)[i - 1] = ri[0];
+    if (i >= 2 && lane < cs) cluster.map_shared_rank(sm, lane)[n + i - 2] = ri[1];
   }
   cluster.sync();
+  // sum of squares of x[1..len) in the order of 512 threads: warps 0 to 15
+  auto partial = [&](const double* x, int len) {
+    if (tid < 512) {
+      double s = 0.0;
+      for (int l = tid; l < len; l += 512)
+        if (l > 0) s = fma(x[l], x[l], s);
+      s = wsum(s);
+      if (lane == 0) red[wid] = s;
+    }
+  };
+  auto scalars = [&](const double* x) {   // warp 0; the two quotients in two lanes
+    double s = (lane < 16) ? red[lane] : 0.0;
+    s = wsum(s);
+    const double x0 = x[0];
+    double tau = 0.0, beta = x0, scale = 0.0;
+    if (s > 0.0) {
+      beta = -copysign(sqrt(fma(x0, x0, s)), x0);
+      const double q = (lane == 1 ? 1.0 : beta - x0) / (lane == 1 ? x0 - beta : beta);
+      tau = __shfl_sync(0xffffffffu, q, 0);
+      scale = __shfl_sync(0xffffffffu, q, 1);
+    }
+    if (lane == 0) {
+      s_tau = tau;
+      s_beta = beta;
+      s_scale = scale;
+    }
+  };
+  partial(sm, n - 1);
+  __syncthreads();
+  if (wid == 0) scalars(sm);
+  __syncthreads();
+  for (int l = tid; l < n - 1; l += SYL_THREADS) sm[l] = (l == 0) ? 1.0 : sm[l] * s_scale;
+  __syncthreads();
+  int rot = 0;                       // b0 = sm + rot n
   for (int j = 0; j < n - 2; ++j) {
     const int len = n - j - 1;
-    // ---- 0: reflector from the broadcast column
-    double s = 0.0;
-    for (int l = threadIdx.x; l < len; l += blockDim.x) {
-      const double x = vn[l];
-      v[l] = x;
-      if (l > 0) s = fma(x, x, s);
-    }
-    s = bsum(s, red);
-    if (threadIdx.x == 0) {
-      const double x0 = v[0];
-      double tau = 0.0, beta = x0, scale = 0.0;
-      if (s > 0.0) {
-        beta = -copysign(sqrt(fma(x0, x0, s)), x0);
-        tau = (beta - x0) / beta;
-        scale = 1.0 / (x0 - beta);
+    const double* v = sm + (size_t)rot * n;
+    const int r1 = (rot == 2) ? 0 : rot + 1, r2 = (r1 == 2) ? 0 : r1 + 1;
+    double* xn = sm + (size_t)r1 * n;
+    double* part = sm + (size_t)r2 * n;
+    const double tau = s_tau, beta = s_beta;
+    // ---- 1: column parts and row parts
+    for (int l = tid; l < len; l += SYL_THREADS) {
+      const int c = j + 1 + l;
+      int sl = (c >= rank) ? (c - rank) / cs + 1 : 0;   // first owned row > c
+      double acc = 0.0;
+      size_t o = sy_off(sl, cs, rank);
+#pragma unroll 4
+      for (int i = sl * cs + rank; i < n; i += cs) {
+        acc = fma(rows[o + c], v[i - j - 1], acc);
+        o += (size_t)i + 1;                          // row i holds i + 1 entries
       }
-      s_tau = tau; s_beta = beta; s_scale = scale;
+      part[l] = acc;
     }
-    __syncthreads();
-    const double tau = s_tau, scale = s_scale;
-    for (int l = 1 + threadIdx.x; l < len; l += blockDim.x) v[l] *= scale;
-    if (threadIdx.x == 0) v[0] = 1.0;
-    __syncthreads();
-    // ---- 1: row parts and column parts
     const int sl0 = (j + 1 > rank) ? (j + 1 - rank + cs - 1) / cs : 0;   // first owned row > j
-    for (int sl = sl0 + wid; sl < slots; sl += wpb) {
+    for (int sl = sl0 + wid; sl < slots; sl += nw) {
       const int i = sl * cs + rank;
       const double* ri = rows + sy_off(sl, cs, rank) + j + 1;
       const int cnt = i - j;                         // c = j + 1 .. i
@@ -784,70 +815,88 @@ __global__ void __launch_bounds__(SY_THREADS) k_sytrd_cluster_lower(int n, doubl
       const double rp = wsum((a0 + a1) + (a2 + a3));
       if (lane == 0) rowp[sl] = rp;
     }
-    for (int l = threadIdx.x; l < len; l += blockDim.x) {
-      const int c = j + 1 + l;
-      int sl = (c >= rank) ? (c - rank) / cs + 1 : 0;   // first owned row > c
-      double acc = 0.0;
-      size_t o = sy_off(sl, cs, rank);
-      for (int i = sl * cs + rank; i < n; i += cs) {
-        acc = fma(rows[o + c], v[i - j - 1], acc);
-        o += (size_t)i + 1;                          // row i holds i + 1 entries
-      }
-      part[l] = acc;
-    }
     cluster.sync();
     // ---- 2: p_i for the owned rows, broadcast
-    double kp = 0.0;
-    for (int sl = sl0 + wid; sl < slots; sl += wpb) {
+    for (int sl = sl0 + wid; sl < slots; sl += nw) {
       const int i = sl * cs + rank;
       const int li = i - j - 1;
       double x = (lane < cs) ? cluster.map_shared_rank(part, lane)[li] : 0.0;
       x = wsum(x);
       const double pi = (rowp[sl] + x) * tau;
       if (lane < cs) cluster.map_shared_rank(p, lane)[li] = pi;
-      if (lane == 0) kp = fma(pi, v[li], kp);
-    }
-    kp = bsum(kp, red);
-    const double kp0 = __shfl_sync(0xffffffffu, kp, 0);
-    if (threadIdx.x < cs) cluster.map_shared_rank(kpart, (int)threadIdx.x)[rank] = kp0;
-    cluster.sync();
-    // ---- 3: update, reflector, next column
-    double K = 0.0;
-    for (int c = 0; c < cs; ++c) K += kpart[c];
-    K *= 0.5 * tau;
-    double* w = part;
-    for (int l = threadIdx.x; l < len; l += blockDim.x) w[l] = p[l] - K * v[l];
-    __syncthreads();
-    for (int sl = sl0 + wid; sl < slots; sl += wpb) {
-      const int i = sl * cs + rank;
-      const int li = i - j - 1;
-      double* ri = rows + sy_off(sl, cs, rank);
-      const double vi = v[li], wi = w[li];
-      const int cnt = i - j;
-      double* rr = ri + j + 1;
-      for (int l = lane; l < cnt; l += 32) rr[l] = fma(-vi, w[l], fma(-wi, v[l], rr[l]));
       __syncwarp();
-      if (lane == 0) ri[j] = vi;                       // reflector entry (row i, column j)
-      if (i > j + 1 && lane < cs) cluster.map_shared_rank(vn, lane)[i - j - 2] = ri[j + 1];
+      if (lane == 0) rowp[sl] = pi;
     }
-    if (threadIdx.x == 0) {
-      if (rank == j % cs) d[j] = rows[sy_off(j / cs, cs, rank) + j];
-      if (rank == 0) {
-        e[j] = s_beta;
-        tauh[j] = tau;
+    __syncthreads();
+    if (wid == 0) {
+      double kp = 0.0;
+      if (lane < 16)
+        for (int sl = sl0 + lane; sl < slots; sl += 16) kp = fma(rowp[sl], v[sl * cs + rank - j - 1], kp);
+      kp = wsum(kp);
+      if (lane < cs) cluster.map_shared_rank(kpart, lane)[rank] = kp;
+    }
+    cluster.sync();
+    // ---- 3: w and the next column
+    if (wid == 0) {
+      double K = 0.0;
+      for (int c = 0; c < cs; ++c) K += kpart[c];
+      K *= 0.5 * tau;
+      if (lane == 0) {
+        s_K = K;
+        s_w0 = p[0] - K * v[0];
       }
     }
-    cluster.sync();
+    __syncthreads();
+    const double K = s_K, w0 = s_w0;
+    for (int l = tid; l < len; l += SYL_THREADS) {
+      const double wl = (l == 0) ? w0 : p[l] - K * v[l];
+      p[l] = wl;
+      if (l > 0) xn[l - 1] = fma(-v[l], w0, fma(-wl, 1.0, xn[l - 1]));
+    }
+    __syncthreads();
+    const bool more = j + 1 < n - 2;
+    if (more) partial(xn, len - 1);
+    __syncthreads();
+    if (wid == 0 && more) scalars(xn);
+    if ((wid & 3) != 0) {
+      const double* w = p;
+      for (int sl = sl0 + (wid >> 2) * 3 + (wid & 3) - 1; sl < slots; sl += nw / 4 * 3) {
+        const int i = sl * cs + rank;
+        const int li = i - j - 1;
+        double* ri = rows + sy_off(sl, cs, rank);
+        const double vi = v[li], wi = w[li];
+        const int cnt = i - j;
+        double* rr = ri + j + 1;
+        for (int l = lane; l < cnt; l += 32) rr[l] = fma(-vi, w[l], fma(-wi, v[l], rr[l]));
+        __syncwarp();
+        if (lane == 0) ri[j] = vi;                       // reflector entry (row i, column j)
+        if (i > j + 2 && lane < cs) cluster.map_shared_rank(part, lane)[i - j - 3] = ri[j + 2];
+      }
+      if (tid == 32) {
+        if (rank == j % cs) d[j] = rows[sy_off(j / cs, cs, rank) + j];
+        if (rank == 0) {
+          e[j] = beta;
+          tauh[j] = tau;
+        }
+      }
+    }
+    __syncthreads();
+    if (more) {
+      const double scale = s_scale;
+      for (int l = tid; l < len - 1; l += SYL_THREADS) xn[l] = (l == 0) ? 1.0 : xn[l] * scale;
+    }
+    __syncthreads();
+    rot = r1;
   }
-  if (threadIdx.x == 0) {
+  if (tid == 0) {
     if (rank == (n - 2) % cs) {
       d[n - 2] = rows[sy_off((n - 2) / cs, cs, rank) + n - 2];
       tauh[n - 2] = 0.0;
     }
     if (rank == (n - 1) % cs) {
-      const double* r1 = rows + sy_off((n - 1) / cs, cs, rank);
-      d[n - 1] = r1[n - 1];
-      e[n - 2] = r1[n - 2];
+      const double* rl = rows + sy_off((n - 1) / cs, cs, rank);
+      d[n - 1] = rl[n - 1];
+      e[n - 2] = rl[n - 2];
       e[n - 1] = 0.0;
       tauh[n - 1] = 0.0;
     }
@@ -855,12 +904,13 @@ __global__ void __launch_bounds__(SY_THREADS) k_sytrd_cluster_lower(int n, doubl
   for (int sl = 0; sl < slots; ++sl) {
     const int i = sl * cs + rank;
     const double* ri = rows + sy_off(sl, cs, rank);
-    for (int c = threadIdx.x; c <= i; c += blockDim.x) {
+    for (int c = tid; c <= i; c += SYL_THREADS) {
       const double x = ri[c];
       A[(size_t)i * lda + c] = x;
       A[(size_t)c * lda + i] = x;
     }
   }
+  cluster.sync();   // no CTA leaves while another may still write into its shared memory
 }
 
 static size_t sytrd_lower_smem_bytes(int n, int cs) {
@@ -929,7 +979,7 @@ static int sytrd_lower_cluster(int n) {
     cudaFuncSetAttribute((const void*)k_sytrd_cluster_lower, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(cs);
-    cfg.blockDim = dim3(SY_THREADS);
+    cfg.blockDim = dim3(SYL_THREADS);
     cfg.dynamicSmemBytes = (size_t)max_optin - 2048;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -1010,7 +1060,7 @@ static sdp_status sytrd(cudaStream_t st, int n, double* A, EigWork* w) {
     if (cs > 0) {
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3(cs);
-      cfg.blockDim = dim3(SY_THREADS);
+      cfg.blockDim = dim3(SYL_THREADS);
       cfg.dynamicSmemBytes = sytrd_lower_smem_bytes(n, cs);
       cfg.stream = st;
       cudaLaunchAttribute at[1];
