@@ -118,10 +118,12 @@ static BDesc make_desc(sdp_problem* h, int active, int prec) {
   D.active = active;
   D.zscale = h->zscale;
   D.inv_tau2 = 1.0 / (h->tau * h->tau);
-  D.rowptr = h->rowptr; D.rowperm = h->rowperm; D.colidx = h->colidx; D.sptr = h->sptr; D.scon = h->scon;
+  D.rowptr = h->rowptr; D.colidx = h->colidx; D.sptr = h->sptr; D.scon = h->scon;
+  D.sellrow = h->sellrow; D.sellcol = h->sellcol; D.sellpos = h->sellpos;
   D.eptr = h->eptr; D.ep = h->ep; D.eq = h->eq;
   D.scoef = h->scoef; D.ecoef = h->ecoef; D.ginv = h->ginv;
   D.W = h->W; D.U = h->U; D.T = h->T; D.Vval = h->Vval;
+  D.Vsell = h->Vsell; D.Vsell32 = h->Vsell32;
   D.pverts = h->hs_pverts; D.rverts = h->hs_rverts; D.btptr = h->hs_btptr; D.btslot = h->hs_btslot;
   D.bp = h->hs_bp; D.bptr = h->hs_bptr; D.bcol = h->hs_bcol;
   D.D = h->hs_D; D.F = h->hs_F; D.Cinv = h->hs_Cinv; D.CinvT = h->hs_CinvT;

@@ -71,10 +71,13 @@ struct BDesc {
   int n, m, k, np, nr, Rk, nnzV;
   int active;                       // the problem's PCG loop is still running
   double zscale, inv_tau2;
-  const int *rowptr, *rowperm, *colidx, *sptr, *scon, *eptr, *ep, *eq;
+  const int *rowptr, *colidx, *sptr, *scon, *eptr, *ep, *eq;
+  const int4* sellrow;
+  const int *sellcol, *sellpos;
   const double *scoef, *ecoef, *ginv;
   const double *W, *U;
-  double *T, *Vval;
+  double *T, *Vval, *Vsell;
+  float* Vsell32;
   const int *pverts, *rverts, *btptr, *btslot, *bp, *bptr, *bcol;
   const double *D, *F, *Cinv, *CinvT;
   double *yP, *v1, *v2, *uvec, *Bn;
@@ -93,6 +96,12 @@ struct BDesc {
   const double *Etop, *wtop;
   double *mvG, *mvQ;
 };
+
+// Threads per block of the Hhat apply's warp-per-row kernels (no block sums): two
+// warps, so that the few hundred rows of one problem reach every SM -- a warp's
+// FP64 instruction holds its scheduler's pipe for 64 cycles, and blocks of eight
+// warps left two thirds of the SMs without one.
+constexpr int HAT_THREADS = 64;
 
 // Finds the problem that owns block b of a batched grid: off[0..N] are the
 // first blocks of each problem (off[N] = total).
@@ -314,8 +323,15 @@ struct sdp_problem {
   // ---- sparse constraint operator (device) ----
   int nnzV = 0;            // CSR pattern of V = sum v_i A_i (both triangles)
   int* rowptr = nullptr;   // n+1
-  int* rowperm = nullptr;  // n   rows by decreasing length (SpMM thread -> row)
   int* colidx = nullptr;   // nnzV
+  // The same entries for the SpMM (sliced ELL): slices of 32 rows by decreasing
+  // length, entry j of a slice's 32 rows side by side, so that a warp whose lanes walk one
+  // row each reads whole lines
+  int4* sellrow = nullptr; // n   row, length, first place, by decreasing length
+  int* sellcol = nullptr;  // column of every place (padding: 0, never read)
+  int* sellpos = nullptr;  // nnzV   slot -> place
+  int* sellcon = nullptr;  // constraint and coefficient of every place, where each slot has one contributor
+  double* sellcoef = nullptr;
   int* sptr = nullptr;     // nnzV+1  slot -> contributors
   int* scon = nullptr;     // contributors: constraint
   double* scoef = nullptr; // contributors: coefficient
@@ -357,6 +373,8 @@ struct sdp_problem {
 
   // ---- matvec work ----
   double* Vval = nullptr;  // nnzV
+  double* Vsell = nullptr; // the values of a Hessian product in the sliced layout
+  float* Vsell32 = nullptr;   // the same in float, for the reduced-precision product
   double* T = nullptr;     // n*n
   float* W32 = nullptr;    // n*n (reduced-precision copies, lazily allocated)
   float* T32 = nullptr;

@@ -43,166 +43,286 @@ __device__ __forceinline__ double wsum_d(double v) {
 __device__ __forceinline__ void assemble_body(int s, int nnzV, const int* __restrict__ sptr,
                                               const int* __restrict__ scon, const double* __restrict__ scoef,
                                               const double* __restrict__ v, const double* __restrict__ scale,
-                                              double* __restrict__ Vval) {
+                                              double* __restrict__ Vval, const int* __restrict__ sellpos,
+                                              double* __restrict__ Vsell, float* __restrict__ Vsell32) {
   if (s >= nnzV) return;
+  const int pos = sellpos ? sellpos[s] : 0;
   double acc = 0.0;
   for (int c = sptr[s]; c < sptr[s + 1]; ++c) {
     const int k = scon[c];
     const double f = scale ? scale[k] : 1.0;
     acc = fma(scoef[c] * f, v[k], acc);
   }
-  Vval[s] = acc;
+  if (Vval) Vval[s] = acc;
+  if (Vsell) Vsell[pos] = acc;
+  if (Vsell32) Vsell32[pos] = (float)acc;
 }
 __global__ void k_assemble(int nnzV, const int* __restrict__ sptr, const int* __restrict__ scon,
                            const double* __restrict__ scoef, const double* __restrict__ v,
-                           const double* __restrict__ scale, double* __restrict__ Vval) {
-  assemble_body(blockIdx.x * blockDim.x + threadIdx.x, nnzV, sptr, scon, scoef, v, scale, Vval);
+                           const double* __restrict__ scale, double* __restrict__ Vval,
+                           const int* __restrict__ sellpos, double* __restrict__ Vsell, float* __restrict__ Vsell32) {
+  assemble_body(blockIdx.x * blockDim.x + threadIdx.x, nnzV, sptr, scon, scoef, v, scale, Vval, sellpos, Vsell,
+                Vsell32);
 }
 
 void assemble_V(sdp_problem* h, const double* v, const double* scale, double* Vval) {
   count_launch();
-  k_assemble<<<cdiv(h->nnzV, 256), 256, 0, h->stream>>>(h->nnzV, h->sptr, h->scon, h->scoef, v, scale, Vval);
+  k_assemble<<<cdiv(h->nnzV, 256), 256, 0, h->stream>>>(h->nnzV, h->sptr, h->scon, h->scoef, v, scale, Vval, nullptr,
+                                                        nullptr, nullptr);
+}
+// V of a Hessian product in the layout of its SpMM; the split form also reads the CSR values.
+static void assemble_matvec(sdp_problem* h, const double* v, bool lp) {
+  count_launch();
+  k_assemble<<<cdiv(h->nnzV, 256), 256, 0, h->stream>>>(h->nnzV, h->sptr, h->scon, h->scoef, v, nullptr,
+                                                        lp ? h->Vval : nullptr, h->sellpos, lp ? nullptr : h->Vsell,
+                                                        lp ? h->Vsell32 : nullptr);
 }
 
 // ---------------------------------------------------------------------------
 // K1: T = W V, R rows of W per CTA staged in shared memory
 // ---------------------------------------------------------------------------
+// A CTA takes R rows of W in shared memory and all rows of V, a warp 32 rows of V (a
+// slice of the sliced-ELL layout, lane = row).  Every entry of T is one thread's sum
+// in the row's CSR order, whatever R and the number of warps.
+//
+// FP64: the FP64 pipe is the bound, one warp instruction per 64 cycles and
+// scheduler, so what counts is that all schedulers get the same number of
+// entries: slices come by decreasing length and are dealt over the four
+// schedulers of the SM (warp number mod 4) there and back, and R is chosen (spmm_rows)
+// so that the CTAs fill whole waves of the SMs.  n = 565, 71250 entries: 128 us with
+// chunks of eight warps, whose CTAs left a third of the SM time idle.
 constexpr int SPMM_UNROLL = 8;
-// FP64: a CTA (SPMM_COLS threads) takes R rows of W and one chunk of SPMM_COLS
-// rows of V: block blk = (row block) * chunks + chunk, so a problem has
-// ceil(n / R) * ceil(n / SPMM_COLS) CTAs -- enough to fill the GPU when only a
-// few problems of a batch are still iterating.  Thread t of chunk c handles
-// row perm[c * SPMM_COLS + t] of V (rows by decreasing length, so that the
-// lanes of a warp walk rows of about the same length).  Every entry of T is
-// one thread's sum in the row's CSR order, whatever R and the chunking.
-constexpr int SPMM_COLS = 256;
-__host__ __device__ __forceinline__ int spmm_chunks(int n) { return (n + SPMM_COLS - 1) / SPMM_COLS; }
+// Slice number it of warp w, of nw (a multiple of 4) warps.
+__device__ __forceinline__ int spmm_slice(int w, int nw, int it) {
+  const int q = (w >> 2) + it * (nw >> 2);
+  return 4 * q + ((q & 1) ? 3 - (w & 3) : (w & 3));
+}
+static int spmm_threads(int n) {
+  const int slices = (n + 31) / 32;
+  return 32 * std::max(4, std::min(16, (slices + 3) / 4 * 4));
+}
 template <int R>
-__device__ __forceinline__ void spmm_f64_body(int blk, int n, const int* __restrict__ rowptr,
-                                              const int* __restrict__ perm, const int* __restrict__ colidx,
-                                              const double* __restrict__ Vval, const double* __restrict__ W,
-                                              double* __restrict__ T, double* wsh) {
-  const int nc = spmm_chunks(n);
-  const int r0 = (blk / nc) * R, t = (blk % nc) * SPMM_COLS + (int)threadIdx.x;
-  for (int e = threadIdx.x; e < R * n; e += blockDim.x) {
-    const int rr = e / n, c = e % n;
-    wsh[e] = (r0 + rr < n) ? W[(size_t)(r0 + rr) * n + c] : 0.0;
-  }
+__device__ __forceinline__ void spmm_f64_body(int blk, int n, const int4* __restrict__ sellrow,
+                                              const int* __restrict__ sellcol, const double* __restrict__ Vsell,
+                                              const double* __restrict__ W, double* __restrict__ T, double* wsh) {
+  const int r0 = blk * R, nw = blockDim.x >> 5, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+  for (int rr = 0; rr < R; ++rr)
+    for (int c = threadIdx.x; c < n; c += blockDim.x)
+      wsh[rr * n + c] = (r0 + rr < n) ? W[(size_t)(r0 + rr) * n + c] : 0.0;
+  int t = spmm_slice(w, nw, 0) * 32 + lane;
+  int4 row = (t < n) ? sellrow[t] : make_int4(0, 0, 0, 0);   // on its way during the staging
   __syncthreads();
-  if (t < n) {
-    const int l = perm[t];
+  for (int it = 0;;) {
+    if (4 * ((w >> 2) + it * (nw >> 2)) * 32 >= n) break;   // no slice of this group of four left
+    const int4 cur = row;
+    const bool on = t < n;
+    t = spmm_slice(w, nw, ++it) * 32 + lane;
+    row = (t < n) ? sellrow[t] : make_int4(0, 0, 0, 0);
+    if (!on) continue;
     double acc[R];
 #pragma unroll
     for (int rr = 0; rr < R; ++rr) acc[rr] = 0.0;
-    const int s1 = rowptr[l + 1];
-    int s = rowptr[l];
-    // eight entries of column l per step: their loads are independent, so each
-    // thread keeps eight L2 requests in flight instead of one
-    for (; s + SPMM_UNROLL <= s1; s += SPMM_UNROLL) {
+    const int len = cur.y;
+    const int* cp = sellcol + cur.z;
+    const double* vp = Vsell + cur.z;
+    // eight entries per step: their loads are independent and go out together (the
+    // other warps' multiply-adds hide them; loading the next eight ahead as well made
+    // the kernel slower where several CTAs share an SM)
+    int s = 0;
+    for (; s + SPMM_UNROLL <= len; s += SPMM_UNROLL) {
       int col[SPMM_UNROLL];
       double val[SPMM_UNROLL];
 #pragma unroll
       for (int u = 0; u < SPMM_UNROLL; ++u) {
-        col[u] = colidx[s + u];
-        val[u] = Vval[s + u];
+        col[u] = cp[32 * (s + u)];
+        val[u] = vp[32 * (s + u)];
       }
 #pragma unroll
       for (int u = 0; u < SPMM_UNROLL; ++u)
 #pragma unroll
         for (int rr = 0; rr < R; ++rr) acc[rr] = fma(val[u], wsh[rr * n + col[u]], acc[rr]);
     }
-    for (; s < s1; ++s) {
-      const double val = Vval[s];
-      const int col = colidx[s];
+    if (s < len) {   // fewer than eight left
+      int col[SPMM_UNROLL];
+      double val[SPMM_UNROLL];
 #pragma unroll
-      for (int rr = 0; rr < R; ++rr) acc[rr] = fma(val, wsh[rr * n + col], acc[rr]);
+      for (int u = 0; u < SPMM_UNROLL - 1; ++u)
+        if (s + u < len) {
+          col[u] = cp[32 * (s + u)];
+          val[u] = vp[32 * (s + u)];
+        }
+#pragma unroll
+      for (int u = 0; u < SPMM_UNROLL - 1; ++u)
+        if (s + u < len) {
+#pragma unroll
+          for (int rr = 0; rr < R; ++rr) acc[rr] = fma(val[u], wsh[rr * n + col[u]], acc[rr]);
+        }
     }
 #pragma unroll
     for (int rr = 0; rr < R; ++rr)
-      if (r0 + rr < n) T[(size_t)(r0 + rr) * n + l] = acc[rr];
+      if (r0 + rr < n) T[(size_t)(r0 + rr) * n + cur.x] = acc[rr];
   }
 }
 template <int R>
-__global__ void __launch_bounds__(256) k_spmm_wv_f64(int n, const int* __restrict__ rowptr,
-                                                     const int* __restrict__ perm,
-                                                     const int* __restrict__ colidx,
-                                                     const double* __restrict__ Vval,
+__global__ void __launch_bounds__(512) k_spmm_wv_f64(int n, const int4* __restrict__ sellrow,
+                                                     const int* __restrict__ sellcol,
+                                                     const double* __restrict__ Vsell,
                                                      const double* __restrict__ W, double* __restrict__ T) {
   extern __shared__ double wsh[];  // R x n
-  spmm_f64_body<R>(blockIdx.x, n, rowptr, perm, colidx, Vval, W, T, wsh);
+  spmm_f64_body<R>(blockIdx.x, n, sellrow, sellcol, Vsell, W, T, wsh);
 }
 
-// Floats per staged column of the reduced-precision SpMM (see spmm_lp_body).
-__host__ __device__ constexpr int spmm_lp_stride(int R) { return (R % 4 == 0) ? R + 4 : R; }
-template <typename TW, int R>
-__device__ __forceinline__ void spmm_lp_body(int blk, int n, const int* __restrict__ rowptr,
-                                             const int* __restrict__ perm, const int* __restrict__ colidx,
-                                             const double* __restrict__ Vval, const TW* __restrict__ W,
-                                             float* __restrict__ T, float* fsh) {
-  // no column chunks here: in FP32 the FMAs are cheap next to staging R rows
-  // of W, so every CTA walks all rows of V for its R rows of W.  The R rows are
-  // staged transposed with a row stride of RS = spmm_lp_stride(R) floats
-  // (fsh[c * RS + rr]): the R values one stored entry of V needs are
-  // contiguous (R / 4 vector loads), and the pad of 4 makes the stride an odd
-  // number of 16-byte groups so that the random columns of a warp's lanes do
-  // not all fall on the same banks (without it the kernel ran 1.4x slower;
-  // with it, as fast as R scattered scalar loads: the CSR loads bound it).
-  // Each acc[rr] sums in the same order as with any other layout.
-  constexpr int RS = spmm_lp_stride(R);
-  const int r0 = blk * R;
-  for (int e = threadIdx.x; e < R * n; e += blockDim.x) {
-    const int rr = e / n, c = e % n;
-    fsh[c * RS + rr] = (r0 + rr < n) ? tof<TW>(W[(size_t)(r0 + rr) * n + c]) : 0.f;
-  }
-  __syncthreads();
-  auto fma_row = [&](float val, int col, float* acc) {
-    const float* w = fsh + col * RS;
-    if constexpr (R % 4 == 0) {
+// The product of small orders, where launches and latency count: the values of V are
+// formed where they are used (every slot has one contributor; the place's
+// constraint and coefficient lie in the sliced layout), so the assembly is no
+// launch of its own.  One row of W per CTA.  n = 40: 12.4 -> 9.9 us for the product.
+constexpr int SPMM_SMALL_N = 192;
+__global__ void __launch_bounds__(256) k_spmm_wv_small(int n, const int4* __restrict__ sellrow,
+                                                       const int* __restrict__ sellcol,
+                                                       const int* __restrict__ sellcon,
+                                                       const double* __restrict__ sellcoef,
+                                                       const double* __restrict__ v, const double* __restrict__ W,
+                                                       double* __restrict__ T) {
+  __shared__ double w[SPMM_SMALL_N];
+  const int r = blockIdx.x, t = threadIdx.x;
+  const int4 row = (t < n) ? sellrow[t] : make_int4(0, 0, 0, 0);
+  if (t < n) w[t] = W[(size_t)r * n + t];
+  double acc = 0.0;
+  for (int s = 0; s < row.y || s == 0; s += SPMM_UNROLL) {
+    int col[SPMM_UNROLL];
+    double val[SPMM_UNROLL];
 #pragma unroll
-      for (int q = 0; q < R / 4; ++q) {
-        const float4 w4 = reinterpret_cast<const float4*>(w)[q];
-        acc[4 * q + 0] = fmaf(val, w4.x, acc[4 * q + 0]);
-        acc[4 * q + 1] = fmaf(val, w4.y, acc[4 * q + 1]);
-        acc[4 * q + 2] = fmaf(val, w4.z, acc[4 * q + 2]);
-        acc[4 * q + 3] = fmaf(val, w4.w, acc[4 * q + 3]);
+    for (int u = 0; u < SPMM_UNROLL; ++u)
+      if (s + u < row.y) {
+        const int e = row.z + 32 * (s + u);
+        col[u] = sellcol[e];
+        val[u] = fma(sellcoef[e], v[sellcon[e]], 0.0);
       }
-    } else {
+    if (s == 0) __syncthreads();
 #pragma unroll
-      for (int rr = 0; rr < R; ++rr) acc[rr] = fmaf(val, w[rr], acc[rr]);
+    for (int u = 0; u < SPMM_UNROLL; ++u)
+      if (s + u < row.y) acc = fma(val[u], w[col[u]], acc);
+  }
+  if (t < n) T[(size_t)r * n + row.x] = acc;
+}
+
+// Reduced precision: the R values of W_s that one stored entry of V needs lie side by
+// side (column-major staging), read by vector loads; they bound the kernel, so bfloat16
+// copies are staged as they are (half the bytes, widened in registers: the same
+// float) and V comes as float from the assembly (a conversion from double holds the
+// FP64 pipe).  Elements per staged column: padded to an odd number of 16-byte groups
+// from 32 bytes on, so that the random columns of a warp's lanes do not all fall on
+// the same banks (without it the float form ran 1.4x slower).
+template <typename TW> __host__ __device__ constexpr int spmm_lp_stride(int R) {
+  return (sizeof(TW) == 4) ? ((R % 4 == 0) ? R + 4 : R) : ((R == 16) ? 24 : R);
+}
+template <typename TW> __host__ __device__ constexpr size_t spmm_lp_bytes(int R) {   // per column of W
+  return sizeof(TW) * spmm_lp_stride<TW>(R);
+}
+__device__ __forceinline__ float bf_lo(uint32_t u) { return __uint_as_float(u << 16); }
+__device__ __forceinline__ float bf_hi(uint32_t u) { return __uint_as_float(u & 0xFFFF0000u); }
+template <typename TW, int R>
+__device__ __forceinline__ void spmm_lp_fma(float val, const TW* w, float* acc) {
+  if constexpr (sizeof(TW) == 4 && R % 4 == 0) {
+#pragma unroll
+    for (int q = 0; q < R / 4; ++q) {
+      const float4 w4 = reinterpret_cast<const float4*>(w)[q];
+      acc[4 * q + 0] = fmaf(val, w4.x, acc[4 * q + 0]);
+      acc[4 * q + 1] = fmaf(val, w4.y, acc[4 * q + 1]);
+      acc[4 * q + 2] = fmaf(val, w4.z, acc[4 * q + 2]);
+      acc[4 * q + 3] = fmaf(val, w4.w, acc[4 * q + 3]);
     }
-  };
-  for (int t = threadIdx.x; t < n; t += blockDim.x) {
-    const int l = perm[t];
+  } else if constexpr (sizeof(TW) == 2 && R % 4 == 0) {
+#pragma unroll
+    for (int q = 0; q < R / 4; q += 2) {
+      uint32_t u[4];
+      if constexpr (R % 8 == 0) {
+        const uint4 x = reinterpret_cast<const uint4*>(w)[q / 2];
+        u[0] = x.x; u[1] = x.y; u[2] = x.z; u[3] = x.w;
+      } else {
+        const uint2 x = reinterpret_cast<const uint2*>(w)[0];
+        u[0] = x.x; u[1] = x.y;
+      }
+#pragma unroll
+      for (int e = 0; e < (R % 8 == 0 ? 4 : 2); ++e) {
+        acc[4 * q + 2 * e] = fmaf(val, bf_lo(u[e]), acc[4 * q + 2 * e]);
+        acc[4 * q + 2 * e + 1] = fmaf(val, bf_hi(u[e]), acc[4 * q + 2 * e + 1]);
+      }
+    }
+  } else {
+#pragma unroll
+    for (int rr = 0; rr < R; ++rr) acc[rr] = fmaf(val, tof<TW>(w[rr]), acc[rr]);
+  }
+}
+template <typename TW, int R>
+__device__ __forceinline__ void spmm_lp_body(int blk, int n, const int4* __restrict__ sellrow,
+                                             const int* __restrict__ sellcol, const float* __restrict__ Vsell,
+                                             const TW* __restrict__ W, float* __restrict__ T, TW* fsh) {
+  constexpr int RS = spmm_lp_stride<TW>(R);
+  const int r0 = blk * R, nw = blockDim.x >> 5, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+  for (int rr = 0; rr < R; ++rr)
+    for (int c = threadIdx.x; c < n; c += blockDim.x)
+      fsh[c * RS + rr] = (r0 + rr < n) ? W[(size_t)(r0 + rr) * n + c] : (TW)0.f;
+  int t = spmm_slice(w, nw, 0) * 32 + lane;
+  int4 row = (t < n) ? sellrow[t] : make_int4(0, 0, 0, 0);   // on its way during the staging
+  __syncthreads();
+  for (int it = 0;;) {
+    if (4 * ((w >> 2) + it * (nw >> 2)) * 32 >= n) break;
+    const int4 cur = row;
+    const bool on = t < n;
+    t = spmm_slice(w, nw, ++it) * 32 + lane;
+    row = (t < n) ? sellrow[t] : make_int4(0, 0, 0, 0);
+    if (!on) continue;
     float acc[R];
 #pragma unroll
     for (int rr = 0; rr < R; ++rr) acc[rr] = 0.f;
-    const int s1 = rowptr[l + 1];
-    int s = rowptr[l];
-    for (; s + SPMM_UNROLL <= s1; s += SPMM_UNROLL) {
-      int col[SPMM_UNROLL];
-      float val[SPMM_UNROLL];
+    const int len = cur.y;
+    const int* cp = sellcol + cur.z;
+    const float* vp = Vsell + cur.z;
+    int col[SPMM_UNROLL];
+    float val[SPMM_UNROLL];
+#pragma unroll
+    for (int u = 0; u < SPMM_UNROLL; ++u) {
+      col[u] = (u < len) ? cp[32 * u] : 0;
+      val[u] = (u < len) ? vp[32 * u] : 0.f;
+    }
+    for (int s = 0; s < len; s += SPMM_UNROLL) {
+      int col1[SPMM_UNROLL];
+      float val1[SPMM_UNROLL];
 #pragma unroll
       for (int u = 0; u < SPMM_UNROLL; ++u) {
-        col[u] = colidx[s + u];
-        val[u] = (float)Vval[s + u];
+        const int e = s + SPMM_UNROLL + u;
+        col1[u] = (e < len) ? cp[32 * e] : 0;
+        val1[u] = (e < len) ? vp[32 * e] : 0.f;
+      }
+      if (s + SPMM_UNROLL <= len) {
+#pragma unroll
+        for (int u = 0; u < SPMM_UNROLL; ++u) spmm_lp_fma<TW, R>(val[u], fsh + col[u] * RS, acc);
+      } else {
+#pragma unroll
+        for (int u = 0; u < SPMM_UNROLL - 1; ++u)
+          if (s + u < len) spmm_lp_fma<TW, R>(val[u], fsh + col[u] * RS, acc);
       }
 #pragma unroll
-      for (int u = 0; u < SPMM_UNROLL; ++u) fma_row(val[u], col[u], acc);
+      for (int u = 0; u < SPMM_UNROLL; ++u) {
+        col[u] = col1[u];
+        val[u] = val1[u];
+      }
     }
-    for (; s < s1; ++s) fma_row((float)Vval[s], colidx[s], acc);
 #pragma unroll
     for (int rr = 0; rr < R; ++rr)
-      if (r0 + rr < n) T[(size_t)(r0 + rr) * n + l] = acc[rr];
+      if (r0 + rr < n) T[(size_t)(r0 + rr) * n + cur.x] = acc[rr];
   }
 }
 template <typename TW, int R>
-__global__ void __launch_bounds__(256) k_spmm_wv_lp(int n, const int* __restrict__ rowptr,
-                                                    const int* __restrict__ perm,
-                                                    const int* __restrict__ colidx,
-                                                    const double* __restrict__ Vval,
+__global__ void __launch_bounds__(512) k_spmm_wv_lp(int n, const int4* __restrict__ sellrow,
+                                                    const int* __restrict__ sellcol,
+                                                    const float* __restrict__ Vsell,
                                                     const TW* __restrict__ W, float* __restrict__ T) {
-  extern __shared__ float fsh[];  // R x n
-  spmm_lp_body<TW, R>(blockIdx.x, n, rowptr, perm, colidx, Vval, W, T, fsh);
+  extern __shared__ __align__(16) unsigned char fsh_raw[];
+  spmm_lp_body<TW, R>(blockIdx.x, n, sellrow, sellcol, Vsell, W, T, reinterpret_cast<TW*>(fsh_raw));
 }
 
 // ---------------------------------------------------------------------------
@@ -288,25 +408,27 @@ __global__ void kb_assemble(const BDesc* __restrict__ desc, const int* __restric
   const BDesc& D = desc[i];
   if (!D.active) return;
   const int lb = blockIdx.x - off[i];
-  assemble_body(lb * blockDim.x + threadIdx.x, D.nnzV, D.sptr, D.scon, D.scoef, D.pp, nullptr, D.Vval);
+  assemble_body(lb * blockDim.x + threadIdx.x, D.nnzV, D.sptr, D.scon, D.scoef, D.pp, nullptr,
+                D.lp ? D.Vval : nullptr, D.sellpos, D.lp ? nullptr : D.Vsell, D.lp ? D.Vsell32 : nullptr);
 }
 // R rows of W per CTA: chosen per batch by the autotuner (batch.cu); every R
 // gives each entry of T by the same sequence of FMAs, so results do not depend on it
 template <int R>
-__global__ void __launch_bounds__(256) kb_spmm(const BDesc* __restrict__ desc, const int* __restrict__ off, int N) {
+__global__ void __launch_bounds__(512) kb_spmm(const BDesc* __restrict__ desc, const int* __restrict__ off, int N) {
   extern __shared__ double wsh[];
   const int i = batch_find(off, N, blockIdx.x);
   const BDesc& D = desc[i];
   if (!D.active || D.lp) return;
-  spmm_f64_body<R>(blockIdx.x - off[i], D.n, D.rowptr, D.rowperm, D.colidx, D.Vval, D.W, D.T, wsh);
+  spmm_f64_body<R>(blockIdx.x - off[i], D.n, D.sellrow, D.sellcol, D.Vsell, D.W, D.T, wsh);
 }
 static void launch_kb_spmm(cudaStream_t st, int R, const BDesc* desc, const int* off, int N, int nb, int nmax) {
   const size_t smem = (size_t)R * nmax * sizeof(double);
+  const int th = spmm_threads(nmax);
   switch (R) {
-    case 1: allow_max_smem((const void*)kb_spmm<1>); kb_spmm<1><<<nb, 256, smem, st>>>(desc, off, N); break;
-    case 2: allow_max_smem((const void*)kb_spmm<2>); kb_spmm<2><<<nb, 256, smem, st>>>(desc, off, N); break;
-    case 8: allow_max_smem((const void*)kb_spmm<8>); kb_spmm<8><<<nb, 256, smem, st>>>(desc, off, N); break;
-    default: allow_max_smem((const void*)kb_spmm<4>); kb_spmm<4><<<nb, 256, smem, st>>>(desc, off, N); break;
+    case 1: allow_max_smem((const void*)kb_spmm<1>); kb_spmm<1><<<nb, th, smem, st>>>(desc, off, N); break;
+    case 2: allow_max_smem((const void*)kb_spmm<2>); kb_spmm<2><<<nb, th, smem, st>>>(desc, off, N); break;
+    case 8: allow_max_smem((const void*)kb_spmm<8>); kb_spmm<8><<<nb, th, smem, st>>>(desc, off, N); break;
+    default: allow_max_smem((const void*)kb_spmm<4>); kb_spmm<4><<<nb, th, smem, st>>>(desc, off, N); break;
   }
 }
 void batch_launch_spmm(cudaStream_t st, int R, const BDesc* desc, const int* off, int N, int nb, int nmax) {
@@ -322,7 +444,7 @@ __global__ void __launch_bounds__(256) kb_sddmm(const BDesc* __restrict__ desc, 
                  D.pp, D.part, D.ticket, D.scal + S_PQ, D.scal + S_RZ, D.scal + S_RZN);
 }
 int batch_blocks_assemble(int nnzV) { return (int)cdiv(nnzV, 256); }
-int batch_blocks_spmm(int n, int R) { return (int)cdiv(n, R) * spmm_chunks(n); }
+int batch_blocks_spmm(int n, int R) { return (int)cdiv(n, R); }
 int batch_blocks_sddmm(int m) { return (int)cdiv(m, SDDMM_PER_BLOCK); }
 // nb_sddmm = 0 leaves the gather out (a mixed batch launches it with the
 // reduced-precision one, batch_launch_sddmm_mixed)
@@ -440,23 +562,36 @@ __global__ void k_split_G(int n, int k, const int* __restrict__ rowptr, const in
 
 // Split: partial sums of (G W_s)[l][q] over a chunk of rows c (FP32; grid.y = chunk)
 constexpr int SPLIT_CHUNKS = 16;
+// The chunk's rows of G as float in shared memory: converted once per block (a
+// conversion from double holds the FP64 pipe as long as a multiply-add; with one per
+// row, term and thread the kernel took three times as long).
+constexpr int SPLIT_STAGE = 64;
 template <typename TW>
 __device__ __forceinline__ void split_R_part_body(int bx, int by, int n, int k, const double* __restrict__ Gt,
                                                   const TW* __restrict__ Ws, float* __restrict__ part) {
+  __shared__ float g[SPLIT_STAGE * 8];
   const int q = bx * blockDim.x + threadIdx.x;
   const int rows = (n + SPLIT_CHUNKS - 1) / SPLIT_CHUNKS;
   const int c0 = by * rows, c1 = min(n, c0 + rows);
-  if (q >= n) return;
   float acc[8];
 #pragma unroll
   for (int l = 0; l < 8; ++l) acc[l] = 0.f;
-#pragma unroll 4
-  for (int c = c0; c < c1; ++c) {
-    const float w = tof<TW>(Ws[(size_t)c * n + q]);
+  for (int cb = c0; cb < c1; cb += SPLIT_STAGE) {
+    const int cnt = min(SPLIT_STAGE, c1 - cb);
+    __syncthreads();
+    for (int t = threadIdx.x; t < cnt * k; t += blockDim.x) g[(t / k) * 8 + t % k] = (float)Gt[(size_t)cb * k + t];
+    __syncthreads();
+    if (q < n) {
+#pragma unroll 8
+      for (int c = 0; c < cnt; ++c) {
+        const float w = tof<TW>(Ws[(size_t)(cb + c) * n + q]);
 #pragma unroll
-    for (int l = 0; l < 8; ++l)
-      if (l < k) acc[l] = fmaf((float)Gt[(size_t)c * k + l], w, acc[l]);
+        for (int l = 0; l < 8; ++l)
+          if (l < k) acc[l] = fmaf(g[c * 8 + l], w, acc[l]);
+      }
+    }
   }
+  if (q >= n) return;
 #pragma unroll
   for (int l = 0; l < 8; ++l)
     if (l < k) part[((size_t)by * k + l) * n + q] = acc[l];
@@ -513,7 +648,7 @@ __global__ void k_split_Ws(int n, int k, const double* __restrict__ W, const dou
 // largest problem fit in 200 KB of shared memory, fewer for larger orders.
 int batch_spmm_lp_rows(int nmax) {
   for (int r = 16; r > 1; r /= 2)
-    if ((size_t)spmm_lp_stride(r) * nmax * sizeof(float) <= 200 * 1024) return r;
+    if (spmm_lp_bytes<float>(r) * nmax <= 200 * 1024) return r;
   return 1;
 }
 __global__ void __launch_bounds__(256) kb_split_G(const BDesc* __restrict__ desc, const int* __restrict__ off, int N) {
@@ -539,17 +674,17 @@ __global__ void __launch_bounds__(256) kb_split_R_Q(const BDesc* __restrict__ de
   split_R_Q_body(blockIdx.x - off[i], D.n, D.ks, D.mvPart, D.wtop, D.mvG, D.Etop, D.mvR, D.mvQ);
 }
 template <int R>
-__global__ void __launch_bounds__(256) kb_spmm_lp(const BDesc* __restrict__ desc, const int* __restrict__ off, int N) {
-  extern __shared__ float fsh[];
+__global__ void __launch_bounds__(512) kb_spmm_lp(const BDesc* __restrict__ desc, const int* __restrict__ off, int N) {
+  extern __shared__ __align__(16) unsigned char fsh_raw[];
   const int i = batch_find(off, N, blockIdx.x);
   const BDesc& D = desc[i];
   if (!D.active || !D.lp) return;
   if (D.bf)
-    spmm_lp_body<__nv_bfloat16, R>(blockIdx.x - off[i], D.n, D.rowptr, D.rowperm, D.colidx, D.Vval,
-                                                 D.W16, D.T32, fsh);
+    spmm_lp_body<__nv_bfloat16, R>(blockIdx.x - off[i], D.n, D.sellrow, D.sellcol, D.Vsell32, D.W16, D.T32,
+                                   reinterpret_cast<__nv_bfloat16*>(fsh_raw));
   else
-    spmm_lp_body<float, R>(blockIdx.x - off[i], D.n, D.rowptr, D.rowperm, D.colidx, D.Vval, D.W32,
-                                         D.T32, fsh);
+    spmm_lp_body<float, R>(blockIdx.x - off[i], D.n, D.sellrow, D.sellcol, D.Vsell32, D.W32, D.T32,
+                           reinterpret_cast<float*>(fsh_raw));
 }
 __global__ void __launch_bounds__(256) kb_sddmm_lp(const BDesc* __restrict__ desc, const int* __restrict__ off,
                                                    int N) {
@@ -597,18 +732,19 @@ void batch_launch_matvec_lp(cudaStream_t st, const BDesc* desc, const int* off_g
                             const int* off_q, const int* off_spmm, const int* off_sddmm, int N, int nb_g, int nb_r,
                             int nb_q, int nb_spmm, int nb_sddmm, int nmax, bool with_sddmm) {
   const int R = batch_spmm_lp_rows(nmax);
-  const size_t smem = (size_t)spmm_lp_stride(R) * nmax * sizeof(float);
+  const size_t smem = spmm_lp_bytes<float>(R) * nmax;   // the bfloat16 staging needs less
+  const int th = spmm_threads(nmax);
   count_launch(with_sddmm ? 5 : 4);
   if (nb_g > 0) kb_split_G<<<nb_g, 256, 0, st>>>(desc, off_g, N);
   if (nb_r > 0) kb_split_R_part<<<nb_r, 128, 0, st>>>(desc, off_r, N);
   if (nb_q > 0) kb_split_R_Q<<<nb_q, 256, 0, st>>>(desc, off_q, N);
   if (nb_spmm > 0) {
     switch (R) {
-      case 16: allow_max_smem((const void*)kb_spmm_lp<16>); kb_spmm_lp<16><<<nb_spmm, 256, smem, st>>>(desc, off_spmm, N); break;
-      case 8: allow_max_smem((const void*)kb_spmm_lp<8>); kb_spmm_lp<8><<<nb_spmm, 256, smem, st>>>(desc, off_spmm, N); break;
-      case 4: allow_max_smem((const void*)kb_spmm_lp<4>); kb_spmm_lp<4><<<nb_spmm, 256, smem, st>>>(desc, off_spmm, N); break;
-      case 2: allow_max_smem((const void*)kb_spmm_lp<2>); kb_spmm_lp<2><<<nb_spmm, 256, smem, st>>>(desc, off_spmm, N); break;
-      default: allow_max_smem((const void*)kb_spmm_lp<1>); kb_spmm_lp<1><<<nb_spmm, 256, smem, st>>>(desc, off_spmm, N); break;
+      case 16: allow_max_smem((const void*)kb_spmm_lp<16>); kb_spmm_lp<16><<<nb_spmm, th, smem, st>>>(desc, off_spmm, N); break;
+      case 8: allow_max_smem((const void*)kb_spmm_lp<8>); kb_spmm_lp<8><<<nb_spmm, th, smem, st>>>(desc, off_spmm, N); break;
+      case 4: allow_max_smem((const void*)kb_spmm_lp<4>); kb_spmm_lp<4><<<nb_spmm, th, smem, st>>>(desc, off_spmm, N); break;
+      case 2: allow_max_smem((const void*)kb_spmm_lp<2>); kb_spmm_lp<2><<<nb_spmm, th, smem, st>>>(desc, off_spmm, N); break;
+      default: allow_max_smem((const void*)kb_spmm_lp<1>); kb_spmm_lp<1><<<nb_spmm, th, smem, st>>>(desc, off_spmm, N); break;
     }
   }
   if (with_sddmm && nb_sddmm > 0) kb_sddmm_lp<<<nb_sddmm, 256, 0, st>>>(desc, off_sddmm, N);
@@ -652,39 +788,72 @@ sdp_status ensure_lowprec_W(sdp_problem* h, int prec) {
   return SDP_OK;
 }
 
-// Rows of W per CTA of the SpMM: as many as shared memory allows (each CTA
-// streams its chunk of the CSR of V once), but few enough that the grid still
-// covers the SMs -- the FP64 form is bound by the SMs' DFMA rate, not by
-// bandwidth.
-static int rows_per_cta(int n, size_t elem) {
+// Rows of W per CTA of the SpMM.  The SM with the most CTAs takes
+// ceil(ceil(n / R) / SMs) of them, each as long as its R multiply-adds and a fixed
+// share per entry (index, value): the R of the least product, at most 200 KB of
+// shared memory.  FP64, 2000 x 2000 with 60000 samples: R = 3, 0.85 ms for the
+// SpMM, 90 % of the FP64 pipe.
+template <typename Bytes>   // bytes(r): staged bytes per column of W
+static int spmm_rows(int n, Bytes bytes, double fixed, const int* cand, int ncand) {
   static int sms = 0;
   if (!sms) {
     int dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   }
-  const size_t budget = 96 * 1024;
-  const int cap = (int)std::min<size_t>(8, budget / (elem * (size_t)n));
-  for (int r = 8; r > 1; r /= 2)
-    if (r <= cap && (n + r - 1) / r >= (sms * 9) / 10) return r;
-  return 1;
+  int best = 1;
+  double tb = 1e300;
+  for (int i = 0; i < ncand; ++i) {
+    const int r = cand[i];
+    if (bytes(r) * (size_t)n > 200 * 1024) continue;
+    const unsigned per_sm = cdiv(cdiv(n, r), sms);
+    const double t = per_sm * (r + fixed) * (per_sm == 1 ? 1.15 : 1.0);   // one CTA alone hides less latency
+    if (t < tb) {
+      tb = t;
+      best = r;
+    }
+  }
+  return best;
 }
 
 template <int R>
-static void launch_spmm_f64(sdp_problem* h, const double* Vval) {
+static void launch_spmm_f64(sdp_problem* h) {
   const size_t smem = (size_t)R * h->n * sizeof(double);
   allow_max_smem((const void*)k_spmm_wv_f64<R>);
   count_launch();
-  k_spmm_wv_f64<R><<<cdiv(h->n, R) * spmm_chunks(h->n), SPMM_COLS, smem, h->stream>>>(h->n, h->rowptr, h->rowperm, h->colidx, Vval, h->W,
-                                                              h->T);
+  k_spmm_wv_f64<R><<<cdiv(h->n, R), spmm_threads(h->n), smem, h->stream>>>(h->n, h->sellrow, h->sellcol, h->Vsell, h->W,
+                                                                           h->T);
+}
+static void spmm_f64(sdp_problem* h) {
+  static const int cand[8] = {8, 7, 6, 5, 4, 3, 2, 1};
+  switch (spmm_rows(h->n, [](int r) { return sizeof(double) * r; }, 0.3, cand, 8)) {
+    case 8: launch_spmm_f64<8>(h); break;
+    case 7: launch_spmm_f64<7>(h); break;
+    case 6: launch_spmm_f64<6>(h); break;
+    case 5: launch_spmm_f64<5>(h); break;
+    case 4: launch_spmm_f64<4>(h); break;
+    case 3: launch_spmm_f64<3>(h); break;
+    case 2: launch_spmm_f64<2>(h); break;
+    default: launch_spmm_f64<1>(h); break;
+  }
 }
 template <typename TW, int R>
-static void launch_spmm_lp(sdp_problem* h, const double* Vval, const TW* W) {
-  const size_t smem = (size_t)spmm_lp_stride(R) * h->n * sizeof(float);
+static void launch_spmm_lp(sdp_problem* h, const TW* W) {
+  const size_t smem = spmm_lp_bytes<TW>(R) * h->n;
   allow_max_smem((const void*)k_spmm_wv_lp<TW, R>);
   count_launch();
-  k_spmm_wv_lp<TW, R><<<cdiv(h->n, R), SPMM_COLS, smem, h->stream>>>(h->n, h->rowptr, h->rowperm, h->colidx, Vval, W,
-                                                                 h->T32);
+  k_spmm_wv_lp<TW, R><<<cdiv(h->n, R), spmm_threads(h->n), smem, h->stream>>>(h->n, h->sellrow, h->sellcol, h->Vsell32, W,
+                                                                              h->T32);
+}
+template <typename TW>
+static void spmm_lp(sdp_problem* h, const TW* W) {
+  static const int cand[4] = {8, 4, 2, 1};
+  switch (spmm_rows(h->n, [](int r) { return spmm_lp_bytes<TW>(r); }, 4.0, cand, 4)) {
+    case 8: launch_spmm_lp<TW, 8>(h, W); break;
+    case 4: launch_spmm_lp<TW, 4>(h, W); break;
+    case 2: launch_spmm_lp<TW, 2>(h, W); break;
+    default: launch_spmm_lp<TW, 1>(h, W); break;
+  }
 }
 
 sdp_status matvec_impl(sdp_problem* h, const double* v, double* Hv, int prec, double* dot_out, double* pro_dst,
@@ -697,19 +866,21 @@ sdp_status matvec_impl(sdp_problem* h, const double* v, double* Hv, int prec, do
   const int n = h->n;
   const bool timed = ktimer_on("matvec");
   if (timed) ktimer_begin(h->stream, "matvec");
-  assemble_V(h, v, nullptr, h->Vval);
   if (prec == SDP_FP64) {
-    switch (rows_per_cta(n, sizeof(double))) {
-      case 8: launch_spmm_f64<8>(h, h->Vval); break;
-      case 4: launch_spmm_f64<4>(h, h->Vval); break;
-      case 2: launch_spmm_f64<2>(h, h->Vval); break;
-      default: launch_spmm_f64<1>(h, h->Vval); break;
+    if (h->sellcon && n <= SPMM_SMALL_N) {
+      count_launch();
+      k_spmm_wv_small<<<n, (n + 31) / 32 * 32, 0, h->stream>>>(n, h->sellrow, h->sellcol, h->sellcon, h->sellcoef, v,
+                                                               h->W, h->T);
+    } else {
+      assemble_matvec(h, v, false);
+      spmm_f64(h);
     }
     count_launch();
     k_sddmm_f64<<<cdiv(h->m, SDDMM_PER_BLOCK), 256, 0, h->stream>>>(n, h->m, h->eptr, h->ep, h->eq, h->ecoef,
                                                                      h->W, h->T, Hv, dv, h->pcg_part,
                                                                      h->pcg_ticket, dot_out, pro_dst, pro_src);
   } else if (prec == SDP_FP32 || prec == SDP_BF16) {
+    assemble_matvec(h, v, true);
     SDP_TRY(ensure_lowprec_W(h, prec));
     const bool split = (prec == SDP_FP32 ? h->W32_key : h->W16_key) >= 0;
     const int ks = split ? h->kpc : 0;
@@ -729,23 +900,13 @@ sdp_status matvec_impl(sdp_problem* h, const double* v, double* Hv, int prec, do
     }
   }
   if (prec == SDP_FP32) {
-    switch (rows_per_cta(n, sizeof(float))) {
-      case 8: launch_spmm_lp<float, 8>(h, h->Vval, h->W32); break;
-      case 4: launch_spmm_lp<float, 4>(h, h->Vval, h->W32); break;
-      case 2: launch_spmm_lp<float, 2>(h, h->Vval, h->W32); break;
-      default: launch_spmm_lp<float, 1>(h, h->Vval, h->W32); break;
-    }
+    spmm_lp<float>(h, h->W32);
     count_launch();
     k_sddmm_lp<float><<<cdiv(h->m, SDDMM_PER_BLOCK), 256, 0, h->stream>>>(
         n, h->m, h->eptr, h->ep, h->eq, h->ecoef, h->W32, h->T32, Hv, dv, h->pcg_part, h->pcg_ticket, dot_out,
         pro_dst, pro_src, h->W32_key >= 0 ? h->kpc : 0, h->Etop, h->mv_R, h->mv_Q);
   } else if (prec == SDP_BF16) {
-    switch (rows_per_cta(n, sizeof(float))) {
-      case 8: launch_spmm_lp<__nv_bfloat16, 8>(h, h->Vval, h->W16); break;
-      case 4: launch_spmm_lp<__nv_bfloat16, 4>(h, h->Vval, h->W16); break;
-      case 2: launch_spmm_lp<__nv_bfloat16, 2>(h, h->Vval, h->W16); break;
-      default: launch_spmm_lp<__nv_bfloat16, 1>(h, h->Vval, h->W16); break;
-    }
+    spmm_lp<__nv_bfloat16>(h, h->W16);
     count_launch();
     k_sddmm_lp<__nv_bfloat16><<<cdiv(h->m, SDDMM_PER_BLOCK), 256, 0, h->stream>>>(
         n, h->m, h->eptr, h->ep, h->eq, h->ecoef, h->W16, h->T32, Hv, dv, h->pcg_part, h->pcg_ticket, dot_out,

@@ -353,8 +353,45 @@ static sdp_status build(sdp_problem* h, int64_t nnzC, const int32_t* Ci, const i
   std::stable_sort(rowperm.begin(), rowperm.end(), [&](int a, int b2) {
     return rowptr[a + 1] - rowptr[a] > rowptr[b2 + 1] - rowptr[b2];
   });
+  const int slices = (n + 31) / 32;
+  std::vector<int4> sellrow(n);
+  std::vector<int> sellpos(std::max(h->nnzV, 1), 0), sellcol;
+  size_t place = 0;
+  for (int sl = 0; sl < slices; ++sl) {
+    const int r0 = rowperm[sl * 32];   // the longest of the slice
+    const size_t width = (size_t)(rowptr[r0 + 1] - rowptr[r0]);
+    sellcol.resize(place + 32 * width, 0);
+    for (int q = 0; q < 32 && sl * 32 + q < n; ++q) {
+      const int r = rowperm[sl * 32 + q];
+      sellrow[sl * 32 + q] = make_int4(r, rowptr[r + 1] - rowptr[r], (int)(place + q), 0);
+      for (int x = rowptr[r]; x < rowptr[r + 1]; ++x) {
+        sellpos[x] = (int)(place + q) + 32 * (x - rowptr[r]);
+        sellcol[sellpos[x]] = colidx[x];
+      }
+    }
+    place += 32 * width;
+  }
+  if (place > (size_t)INT32_MAX) {
+    h->last_error = "sdp_setup: constraint pattern too large";
+    return SDP_ERR_ARG;
+  }
+  if (sellcol.empty()) sellcol.push_back(0);
+  if (h->ncontrib == h->nnzV) {
+    std::vector<int> sellcon(sellcol.size(), 0);
+    std::vector<double> sellcoef(sellcol.size(), 0.0);
+    for (int x = 0; x < h->nnzV; ++x) {
+      sellcon[sellpos[x]] = scon[x];
+      sellcoef[sellpos[x]] = scoef[x];
+    }
+    SDP_TRY(upload(h, &h->sellcon, sellcon));
+    SDP_TRY(upload(h, &h->sellcoef, sellcoef));
+  }
   SDP_TRY(upload(h, &h->rowptr, rowptr));
-  SDP_TRY(upload(h, &h->rowperm, rowperm));
+  SDP_TRY(upload(h, &h->sellrow, sellrow));
+  SDP_TRY(upload(h, &h->sellcol, sellcol));
+  SDP_TRY(upload(h, &h->sellpos, sellpos));
+  SDP_TRY(h->allocT(&h->Vsell, sellcol.size()));
+  SDP_TRY(h->allocT(&h->Vsell32, sellcol.size()));
   SDP_TRY(upload(h, &h->colidx, colidx));
   SDP_TRY(upload(h, &h->sptr, sptr));
   SDP_TRY(upload(h, &h->scon, scon));
