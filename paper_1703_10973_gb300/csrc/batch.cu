@@ -31,10 +31,8 @@
 
 namespace sdpgb {
 
-static inline int cdivi(int a, int b) { return (a + b - 1) / b; }
 
-enum { BK_ASM, BK_SPMM, BK_SDDMM, BK_VEC, BK_HATU, BK_TAIL, BK_FWDP, BK_FWDR, BK_GEMV, BK_OUTR, BK_BWDP,
-       BK_SPLG, BK_SPLR, BK_SPLQ, BK_SPMM_LP, BK_COUNT };
+enum { BK_ASM, BK_SPMM, BK_SDDMM, BK_VEC, BK_HATU, BK_TAIL, BK_FWDR, BK_GEMV, BK_OUT, BK_SPLG, BK_SPLR, BK_SPLQ, BK_SPMM_LP, BK_COUNT };
 
 }  // namespace sdpgb
 
@@ -99,9 +97,8 @@ static void batch_offsets(sdp_batch* b) {
     const int k = std::min(h->kcap, h->n - 1), Rk = h->hs_nr * k;   // grids for the largest rank
     const int cnt[BK_COUNT] = {batch_blocks_assemble(h->nnzV), batch_blocks_spmm(h->n, b->spmm_r), batch_blocks_sddmm(h->m),
                                batch_blocks_vec(h->m),         batch_blocks_hat_u(h->n), batch_blocks_tail(h->m),
-                               batch_blocks_fwdP(h->hs_np),    batch_blocks_warp_rows(h->hs_nr),
-                               batch_blocks_warp_rows(Rk),     batch_blocks_out_bwd(Rk, h->hs_np),
-                               0,
+                               batch_blocks_warp_rows(Rk),     batch_blocks_warp_rows(Rk),
+                               batch_blocks_out_bwd(Rk, h->hs_np),
                                batch_blocks_split_G(h->n),     batch_blocks_split_R(h->n),
                                batch_blocks_split_Q(h->n, k),  batch_blocks_spmm_lp(h->n, b->nmax)};
     for (int kd = 0; kd < BK_COUNT; ++kd)
@@ -116,15 +113,16 @@ static BDesc make_desc(sdp_problem* h, int active, int prec) {
   D.n = h->n; D.m = h->m; D.k = h->kpc; D.np = h->hs_np; D.nr = h->hs_nr; D.Rk = h->hs_nr * h->kpc;
   D.nnzV = h->nnzV;
   D.active = active;
+  D.single = h->single ? 1 : 0;
   D.zscale = h->zscale;
   D.inv_tau2 = 1.0 / (h->tau * h->tau);
   D.rowptr = h->rowptr; D.colidx = h->colidx; D.sptr = h->sptr; D.scon = h->scon;
   D.sellrow = h->sellrow; D.sellcol = h->sellcol; D.sellpos = h->sellpos;
   D.eptr = h->eptr; D.ep = h->ep; D.eq = h->eq;
-  D.scoef = h->scoef; D.ecoef = h->ecoef; D.ginv = h->ginv;
+  D.scoef = h->scoef; D.sg = h->sg; D.ecoef = h->ecoef; D.ginv = h->ginv;
   D.W = h->W; D.U = h->U; D.T = h->T; D.Vval = h->Vval;
   D.Vsell = h->Vsell; D.Vsell32 = h->Vsell32;
-  D.pverts = h->hs_pverts; D.rverts = h->hs_rverts; D.btptr = h->hs_btptr; D.btslot = h->hs_btslot;
+  D.pidx = h->hs_pidx; D.pverts = h->hs_pverts; D.rverts = h->hs_rverts; D.btptr = h->hs_btptr; D.btslot = h->hs_btslot;
   D.bp = h->hs_bp; D.bptr = h->hs_bptr; D.bcol = h->hs_bcol;
   D.D = h->hs_D; D.F = h->hs_F; D.Cinv = h->hs_Cinv; D.CinvT = h->hs_CinvT;
   D.yP = h->hs_yP; D.v1 = h->hs_v1; D.v2 = h->hs_v2; D.uvec = h->uvec; D.Bn = h->Bn;
@@ -190,9 +188,8 @@ static void batch_body(sdp_batch* b, cudaStream_t st, cudaGraphConditionalHandle
   }
   batch_launch_xr(st, b->ddesc, off(BK_VEC), N, b->total[BK_VEC]);
   batch_launch_hat_u(st, b->ddesc, off(BK_HATU), N, b->total[BK_HATU]);
-  batch_launch_core_solve(st, b->ddesc, N, off(BK_FWDP), b->total[BK_FWDP], off(BK_FWDR), b->total[BK_FWDR],
-                          off(BK_GEMV), b->total[BK_GEMV], off(BK_OUTR), b->total[BK_OUTR], off(BK_BWDP),
-                          b->total[BK_BWDP]);
+  batch_launch_core_solve(st, b->ddesc, N, off(BK_FWDR), b->total[BK_FWDR], off(BK_GEMV), b->total[BK_GEMV],
+                          off(BK_OUT), b->total[BK_OUT]);
   batch_launch_tail(st, b->ddesc, off(BK_TAIL), N, b->total[BK_TAIL]);
   batch_launch_p(st, b->ddesc, off(BK_VEC), N, b->total[BK_VEC], cond, flag);
 }

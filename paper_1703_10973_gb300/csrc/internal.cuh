@@ -70,14 +70,16 @@ enum { S_PQ = 0, S_RR = 1, S_RZ = 2, S_RZN = 3, S_TMP = 4, S_NR0 = 5, S_TOL2 = 6
 struct BDesc {
   int n, m, k, np, nr, Rk, nnzV;
   int active;                       // the problem's PCG loop is still running
+  int single;                       // every slot of V has one contributor
   double zscale, inv_tau2;
   const int *rowptr, *colidx, *sptr, *scon, *eptr, *ep, *eq;
   const int4* sellrow;
   const int *sellcol, *sellpos;
-  const double *scoef, *ecoef, *ginv;
+  const double *scoef, *sg, *ecoef, *ginv;
   const double *W, *U;
   double *T, *Vval, *Vsell;
   float* Vsell32;
+  const int *pidx;                  // row -> position in the independent set, -1 for the other rows
   const int *pverts, *rverts, *btptr, *btslot, *bp, *bptr, *bcol;
   const double *D, *F, *Cinv, *CinvT;
   double *yP, *v1, *v2, *uvec, *Bn;
@@ -97,10 +99,8 @@ struct BDesc {
   double *mvG, *mvQ;
 };
 
-// Threads per block of the Hhat apply's warp-per-row kernels (no block sums): two
-// warps, so that the few hundred rows of one problem reach every SM -- a warp's
-// FP64 instruction holds its scheduler's pipe for 64 cycles, and blocks of eight
-// warps left two thirds of the SMs without one.
+// Threads per block of the Hhat apply's warp-per-sum kernels (no block sums): two
+// warps, so that the few hundred sums of one problem reach every SM.
 constexpr int HAT_THREADS = 64;
 
 // Finds the problem that owns block b of a batched grid: off[0..N] are the
@@ -286,6 +286,7 @@ struct SchurPlanHost {
 };
 void schur_plan(int n, const std::vector<int>& krowptr, const std::vector<int>& kcol, SchurPlanHost* out);
 sdp_status schur_build(sdp_problem* h, int k, double tau);
+// y_P already holds L_P^{-1} u_P for k <= 8 (formed with u, precond.cu)
 sdp_status schur_apply(sdp_problem* h, const double* u, double* out, double scale, int prec = SDP_FP64);
 // FP32 copy of the Hhat core's dense factor inverse for applies in reduced precision
 sdp_status ensure_lowprec_core(sdp_problem* h);
@@ -335,6 +336,8 @@ struct sdp_problem {
   int* sptr = nullptr;     // nnzV+1  slot -> contributors
   int* scon = nullptr;     // contributors: constraint
   double* scoef = nullptr; // contributors: coefficient
+  double* sg = nullptr;    // contributors: coefficient / ||A_i||^2
+  bool single = false;     // every slot has one contributor (contributor s belongs to slot s)
   int ncontrib = 0;
   int nent = 0;            // stored upper entries over all constraints
   int* eptr = nullptr;     // m+1   constraint -> entries
@@ -414,6 +417,7 @@ struct sdp_problem {
   // sparse Hhat core (schur.cu): independent set P of the K graph, rest R
   int hs_np = 0, hs_nr = 0, hs_nb = 0, hs_k = 0;
   int *hs_pverts = nullptr, *hs_rverts = nullptr;        // np, nr
+  int* hs_pidx = nullptr;                                // n: position in pverts, -1 for rows of rverts
   int *hs_stype = nullptr, *hs_sa = nullptr, *hs_sb = nullptr;   // per K slot
   int *hs_bptr = nullptr, *hs_bcol = nullptr, *hs_bp = nullptr;  // B blocks by row of P
   int *hs_btptr = nullptr, *hs_btslot = nullptr;         // B blocks by row of R
@@ -515,9 +519,7 @@ int batch_blocks_sddmm(int m);
 int batch_blocks_vec(int m);
 int batch_blocks_hat_u(int n);
 int batch_blocks_tail(int m);
-int batch_blocks_fwdP(int np);
 int batch_blocks_warp_rows(int rows);
-int batch_blocks_outR(int Rk);
 int batch_blocks_out_bwd(int Rk, int np);
 int batch_blocks_split_G(int n);
 int batch_blocks_split_R(int n);
@@ -537,9 +539,8 @@ void batch_launch_p(cudaStream_t st, const BDesc* desc, const int* off, int N, i
 void batch_launch_sddmm_mixed(cudaStream_t st, const BDesc* desc, const int* off, int N, int nb);
 void batch_launch_hat_u(cudaStream_t st, const BDesc* desc, const int* off, int N, int nb);
 void batch_launch_tail(cudaStream_t st, const BDesc* desc, const int* off, int N, int nb);
-void batch_launch_core_solve(cudaStream_t st, const BDesc* desc, int N, const int* off_fwdP, int nb_fwdP,
-                             const int* off_fwdR, int nb_fwdR, const int* off_gemv, int nb_gemv,
-                             const int* off_outR, int nb_outR, const int* off_bwdP, int nb_bwdP);
+void batch_launch_core_solve(cudaStream_t st, const BDesc* desc, int N, const int* off_fwdR, int nb_fwdR,
+                             const int* off_gemv, int nb_gemv, const int* off_out, int nb_out);
 // Restarted PCG as a state machine (pcg.cu), shared by single solves and batches
 struct PcgSweeps {
   const double* r = nullptr;

@@ -40,7 +40,7 @@ __device__ __forceinline__ double wsum_d(double v) {
 // ---------------------------------------------------------------------------
 // K0: V values from v (gather form, no atomics)
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void assemble_body(int s, int nnzV, const int* __restrict__ sptr,
+__device__ __forceinline__ void assemble_body(int s, int nnzV, bool single, const int* __restrict__ sptr,
                                               const int* __restrict__ scon, const double* __restrict__ scoef,
                                               const double* __restrict__ v, const double* __restrict__ scale,
                                               double* __restrict__ Vval, const int* __restrict__ sellpos,
@@ -48,7 +48,8 @@ __device__ __forceinline__ void assemble_body(int s, int nnzV, const int* __rest
   if (s >= nnzV) return;
   const int pos = sellpos ? sellpos[s] : 0;
   double acc = 0.0;
-  for (int c = sptr[s]; c < sptr[s + 1]; ++c) {
+  const int c0 = single ? s : sptr[s], c1 = single ? s + 1 : sptr[s + 1];   // one contributor: no list to look up
+  for (int c = c0; c < c1; ++c) {
     const int k = scon[c];
     const double f = scale ? scale[k] : 1.0;
     acc = fma(scoef[c] * f, v[k], acc);
@@ -57,23 +58,23 @@ __device__ __forceinline__ void assemble_body(int s, int nnzV, const int* __rest
   if (Vsell) Vsell[pos] = acc;
   if (Vsell32) Vsell32[pos] = (float)acc;
 }
-__global__ void k_assemble(int nnzV, const int* __restrict__ sptr, const int* __restrict__ scon,
+__global__ void k_assemble(int nnzV, bool single, const int* __restrict__ sptr, const int* __restrict__ scon,
                            const double* __restrict__ scoef, const double* __restrict__ v,
                            const double* __restrict__ scale, double* __restrict__ Vval,
                            const int* __restrict__ sellpos, double* __restrict__ Vsell, float* __restrict__ Vsell32) {
-  assemble_body(blockIdx.x * blockDim.x + threadIdx.x, nnzV, sptr, scon, scoef, v, scale, Vval, sellpos, Vsell,
+  assemble_body(blockIdx.x * blockDim.x + threadIdx.x, nnzV, single, sptr, scon, scoef, v, scale, Vval, sellpos, Vsell,
                 Vsell32);
 }
 
 void assemble_V(sdp_problem* h, const double* v, const double* scale, double* Vval) {
   count_launch();
-  k_assemble<<<cdiv(h->nnzV, 256), 256, 0, h->stream>>>(h->nnzV, h->sptr, h->scon, h->scoef, v, scale, Vval, nullptr,
+  k_assemble<<<cdiv(h->nnzV, 256), 256, 0, h->stream>>>(h->nnzV, h->single, h->sptr, h->scon, h->scoef, v, scale, Vval, nullptr,
                                                         nullptr, nullptr);
 }
 // V of a Hessian product in the layout of its SpMM; the split form also reads the CSR values.
 static void assemble_matvec(sdp_problem* h, const double* v, bool lp) {
   count_launch();
-  k_assemble<<<cdiv(h->nnzV, 256), 256, 0, h->stream>>>(h->nnzV, h->sptr, h->scon, h->scoef, v, nullptr,
+  k_assemble<<<cdiv(h->nnzV, 256), 256, 0, h->stream>>>(h->nnzV, h->single, h->sptr, h->scon, h->scoef, v, nullptr,
                                                         lp ? h->Vval : nullptr, h->sellpos, lp ? nullptr : h->Vsell,
                                                         lp ? h->Vsell32 : nullptr);
 }
@@ -408,7 +409,7 @@ __global__ void kb_assemble(const BDesc* __restrict__ desc, const int* __restric
   const BDesc& D = desc[i];
   if (!D.active) return;
   const int lb = blockIdx.x - off[i];
-  assemble_body(lb * blockDim.x + threadIdx.x, D.nnzV, D.sptr, D.scon, D.scoef, D.pp, nullptr,
+  assemble_body(lb * blockDim.x + threadIdx.x, D.nnzV, D.single != 0, D.sptr, D.scon, D.scoef, D.pp, nullptr,
                 D.lp ? D.Vval : nullptr, D.sellpos, D.lp ? nullptr : D.Vsell, D.lp ? D.Vsell32 : nullptr);
 }
 // R rows of W per CTA: chosen per batch by the autotuner (batch.cu); every R

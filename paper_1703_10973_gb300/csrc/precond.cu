@@ -22,6 +22,7 @@
 // core has condition number ~ (lambda_max(W) / tau)^2, beyond FP64 once
 // mu ~ 1e-5, while the Hhat core stays near lambda_max(W) / tau.
 #include "internal.cuh"
+#include "rounded.cuh"
 
 #include <algorithm>
 #include <cmath>
@@ -123,42 +124,68 @@ __global__ void k_apply_tail(int m, int k, const int* __restrict__ eptr, const i
 }
 
 // Hhat apply, first product: u[l n + a] = scale * sum_{s in row a} V_s U[col(s)][l]
-// with V = sum_i g_i^{-1} r_i A_i assembled on the fly; one warp per row a.
-__device__ __forceinline__ void hat_u_body(int a, int lane, int n, int k, const int* __restrict__ rowptr,
+// with V = sum_i g_i^{-1} r_i A_i assembled on the fly; one warp per row a.  For a row
+// of the independent set the warp goes on to y_a = L_a^{-1} u_a (the first
+// substitution of the core solve).  sg = coefficient / ||A_i||^2 is laid out once; with
+// one contributor per slot its list is the slot's own number and four slots per lane
+// are in flight.  Bound by those gathers' latency.
+__device__ __forceinline__ void hat_u_body(int a, int lane, int n, int k, bool single, const int* __restrict__ rowptr,
                                            const int* __restrict__ colidx, const int* __restrict__ sptr,
-                                           const int* __restrict__ scon, const double* __restrict__ scoef,
-                                           const double* __restrict__ ginv, const double* __restrict__ r,
-                                           const double* __restrict__ U, double scale, double* __restrict__ u) {
+                                           const int* __restrict__ scon, const double* __restrict__ sg,
+                                           const double* __restrict__ r, const double* __restrict__ U, double scale,
+                                           double* __restrict__ u, const int* __restrict__ pidx,
+                                           const double* __restrict__ D, double* __restrict__ yP) {
   if (a >= n) return;
   double acc[8];
 #pragma unroll
   for (int l = 0; l < 8; ++l) acc[l] = 0.0;
-  for (int s = rowptr[a] + lane; s < rowptr[a + 1]; s += 32) {
-    double v = 0.0;
-    for (int c = sptr[s]; c < sptr[s + 1]; ++c) {
-      const int i = scon[c];
-      v = fma(scoef[c] * ginv[i], r[i], v);
-    }
-    const double* ur = U + (size_t)colidx[s] * k;
+  const int s1 = rowptr[a + 1];
+  const int pa = pidx[a];
+  if (single) {
+#pragma unroll 4
+    for (int s = rowptr[a] + lane; s < s1; s += 32) {
+      const double v = fma(sg[s], r[scon[s]], 0.0);
+      const double* ur = U + (size_t)colidx[s] * k;
 #pragma unroll
-    for (int l = 0; l < 8; ++l)
-      if (l < k) acc[l] = fma(v, ur[l], acc[l]);
+      for (int l = 0; l < 8; ++l)
+        if (l < k) acc[l] = fma(v, ur[l], acc[l]);
+    }
+  } else {
+    for (int s = rowptr[a] + lane; s < s1; s += 32) {
+      double v = 0.0;
+      for (int c = sptr[s]; c < sptr[s + 1]; ++c) v = fma(sg[c], r[scon[c]], v);
+      const double* ur = U + (size_t)colidx[s] * k;
+#pragma unroll
+      for (int l = 0; l < 8; ++l)
+        if (l < k) acc[l] = fma(v, ur[l], acc[l]);
+    }
   }
+  double x[8];
+  const double* La = D + (size_t)(pa < 0 ? 0 : pa) * k * k;
 #pragma unroll
   for (int l = 0; l < 8; ++l) {
     if (l >= k) break;
     double t = acc[l];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    if (lane == 0) u[(size_t)l * n + a] = scale * t;
+    t = scale * t;
+    if (lane == 0) u[(size_t)l * n + a] = t;
+    if (pa >= 0) {
+      double s = t;
+#pragma unroll
+      for (int j = 0; j < l; ++j) s -= La[l * k + j] * x[j];
+      x[l] = div_rn(s, La[l * k + l]);
+      if (lane == 0) yP[(size_t)pa * k + l] = x[l];
+    }
   }
 }
-__global__ void k_hat_u(int n, int k, const int* __restrict__ rowptr, const int* __restrict__ colidx,
-                        const int* __restrict__ sptr, const int* __restrict__ scon, const double* __restrict__ scoef,
-                        const double* __restrict__ ginv, const double* __restrict__ r, const double* __restrict__ U,
-                        double scale, double* __restrict__ u) {
-  hat_u_body((blockIdx.x * blockDim.x + threadIdx.x) >> 5, threadIdx.x & 31, n, k, rowptr, colidx, sptr, scon,
-             scoef, ginv, r, U, scale, u);
+__global__ void k_hat_u(int n, int k, bool single, const int* __restrict__ rowptr, const int* __restrict__ colidx,
+                        const int* __restrict__ sptr, const int* __restrict__ scon, const double* __restrict__ sg,
+                        const double* __restrict__ r, const double* __restrict__ U, double scale,
+                        double* __restrict__ u, const int* __restrict__ pidx, const double* __restrict__ D,
+                        double* __restrict__ yP) {
+  hat_u_body((blockIdx.x * blockDim.x + threadIdx.x) >> 5, threadIdx.x & 31, n, k, single, rowptr, colidx, sptr, scon,
+             sg, r, U, scale, u, pidx, D, yP);
 }
 
 // The same product for split ranks above 8 (up to 64): one warp per row a; the
@@ -203,8 +230,8 @@ __global__ void kb_hat_u(const BDesc* __restrict__ desc, const int* __restrict__
   const BDesc& D = desc[i];
   if (!D.active) return;
   const int lb = blockIdx.x - off[i];
-  hat_u_body((lb * blockDim.x + threadIdx.x) >> 5, threadIdx.x & 31, D.n, D.k, D.rowptr, D.colidx, D.sptr, D.scon,
-             D.scoef, D.ginv, D.pr, D.U, D.zscale, D.uvec);
+  hat_u_body((lb * blockDim.x + threadIdx.x) >> 5, threadIdx.x & 31, D.n, D.k, D.single != 0, D.rowptr, D.colidx, D.sptr,
+             D.scon, D.sg, D.pr, D.U, D.zscale, D.uvec, D.pidx, D.D, D.yP);
 }
 __global__ void kb_apply_tail(const BDesc* __restrict__ desc, const int* __restrict__ off, int N) {
   const int i = batch_find(off, N, blockIdx.x);
@@ -213,11 +240,11 @@ __global__ void kb_apply_tail(const BDesc* __restrict__ desc, const int* __restr
   apply_tail_body(blockIdx.x - off[i], off[i + 1] - off[i], D.m, D.k, D.eptr, D.ep, D.eq, D.ecoef, D.Bn, D.U,
                   D.ginv, D.pr, D.inv_tau2, D.pz, D.part, D.ticket, D.scal + S_RZN);
 }
-int batch_blocks_hat_u(int n) { return (int)cdiv((size_t)n * 32, 256); }
+int batch_blocks_hat_u(int n) { return (int)cdiv((size_t)n * 32, HAT_THREADS); }
 int batch_blocks_tail(int m) { return (int)cdiv(m, 256); }
 void batch_launch_hat_u(cudaStream_t st, const BDesc* desc, const int* off, int N, int nb) {
   count_launch();
-  if (nb > 0) kb_hat_u<<<nb, 256, 0, st>>>(desc, off, N);
+  if (nb > 0) kb_hat_u<<<nb, HAT_THREADS, 0, st>>>(desc, off, N);
 }
 void batch_launch_tail(cudaStream_t st, const BDesc* desc, const int* off, int N, int nb) {
   count_launch();
@@ -643,8 +670,9 @@ sdp_status precond_apply_impl(sdp_problem* h, const double* r, double* z, int pr
       k_hat_u_gen<<<cdiv((size_t)n * 32, 256), 256, 0, st>>>(n, k, h->rowptr, h->colidx, h->sptr, h->scon,
                                                              h->scoef, h->ginv, r, h->U, h->zscale, h->uvec);
     else
-      k_hat_u<<<cdiv((size_t)n * 32, 256), 256, 0, st>>>(n, k, h->rowptr, h->colidx, h->sptr, h->scon, h->scoef,
-                                                         h->ginv, r, h->U, h->zscale, h->uvec);
+      k_hat_u<<<cdiv((size_t)n * 32, HAT_THREADS), HAT_THREADS, 0, st>>>(n, k, h->single, h->rowptr, h->colidx, h->sptr,
+                                                                                 h->scon, h->sg, r, h->U, h->zscale,
+                                                                                 h->uvec, h->hs_pidx, h->hs_D, h->hs_yP);
     SDP_TRY(schur_apply(h, h->uvec, h->Bn, h->zscale, prec));
   } else {
     // u = Z^T (sum g_i r_i A_i) U, stored as k x n (row l = column l of u)

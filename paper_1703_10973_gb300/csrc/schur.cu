@@ -19,6 +19,7 @@
 // The two dense triangular solves use L_C^{-1} with one refinement step
 // against L_C, as the dense core does.
 #include "internal.cuh"
+#include "rounded.cuh"
 
 #include <algorithm>
 #include <cmath>
@@ -241,62 +242,46 @@ __global__ void __launch_bounds__(256) k_hat_schur_rows(int k, int Rk, const int
 // ---------------------------------------------------------------------------
 // Device: apply pieces (u and the result in the k x n layout u[l n + c])
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void fwdP_body(int a, int np, int n, int k, const int* __restrict__ pverts,
-                                          const double* __restrict__ D, const double* __restrict__ u,
-                                          double* __restrict__ yP) {
-  if (a >= np) return;
-  const double* La = D + (size_t)a * k * k;
-  const int v = pverts[a];
-  double x[KMAX];
-  for (int i = 0; i < k; ++i) {
-    double s = u[(size_t)i * n + v];
-    for (int j = 0; j < i; ++j) s -= La[i * k + j] * x[j];
-    x[i] = s / La[i * k + i];
-    yP[(size_t)a * k + i] = x[i];
-  }
-}
-__global__ void k_hat_fwdP(int np, int n, int k, const int* __restrict__ pverts, const double* __restrict__ D,
-                           const double* __restrict__ u, double* __restrict__ yP) {
-  fwdP_body(blockIdx.x * blockDim.x + threadIdx.x, np, n, k, pverts, D, u, yP);
-}
-
 __device__ __forceinline__ double hs_warp_sum(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
 
-// tR[r k + l2] = u[l2 n + rverts[r]] - sum over blocks (a, r) of (F^T y_a)[l2];
-// one warp per r, lanes over the blocks
-__device__ __forceinline__ void fwdR_body(int r, int lane, int nr, int n, int k, const int* __restrict__ rverts,
+// tR[r k + c] = u[c n + rverts[r]] - sum over blocks (a, r) of (F^T y_a)[c]; one
+// warp per (r, c), lanes over the blocks (a warp per r with its k sums spent most of
+// its time waiting for one gather after the other)
+__device__ __forceinline__ void fwdR_body(int wr, int lane, int nr, int n, int k, const int* __restrict__ rverts,
                                           const int* __restrict__ btptr, const int* __restrict__ btslot,
                                           const int* __restrict__ bp, const double* __restrict__ F,
                                           const double* __restrict__ yP, const double* __restrict__ u,
                                           double* __restrict__ tR, float* __restrict__ tRf = nullptr) {
+  if (k == 0) return;   // an adaptive rank of zero: no core
+  const int r = wr / k, c = wr - r * k;
   if (r >= nr) return;
-  double acc[KMAX];
-#pragma unroll
-  for (int c = 0; c < KMAX; ++c) acc[c] = 0.0;
-  for (int e = btptr[r] + lane; e < btptr[r + 1]; e += 32) {
+  double acc = 0.0;
+  const int e1 = btptr[r + 1];
+#pragma unroll 2
+  for (int e = btptr[r] + lane; e < e1; e += 32) {
     const int bi = btslot[e];
-    const double* Fb = F + (size_t)bi * k * k;
+    const double* Fb = F + (size_t)bi * k * k + c;
     const double* ya = yP + (size_t)bp[bi] * k;
-    for (int i = 0; i < k; ++i) {
-      const double yi = ya[i];
+    double f[KMAX], y[KMAX];
 #pragma unroll
-      for (int c = 0; c < KMAX; ++c)
-        if (c < k) acc[c] = fma(Fb[i * k + c], yi, acc[c]);
-    }
+    for (int i = 0; i < KMAX; ++i)
+      if (i < k) {
+        f[i] = Fb[i * k];
+        y[i] = ya[i];
+      }
+#pragma unroll
+    for (int i = 0; i < KMAX; ++i)
+      if (i < k) acc = fma(f[i], y[i], acc);
   }
-#pragma unroll
-  for (int c = 0; c < KMAX; ++c) {
-    if (c >= k) break;
-    const double s = hs_warp_sum(acc[c]);
-    if (lane == 0) {
-      const double t = u[(size_t)c * n + rverts[r]] - s;
-      tR[(size_t)r * k + c] = t;
-      if (tRf) tRf[(size_t)r * k + c] = (float)t;
-    }
+  const double s = hs_warp_sum(acc);
+  if (lane == 0) {
+    const double t = u[(size_t)c * n + rverts[r]] - s;
+    tR[(size_t)r * k + c] = t;
+    if (tRf) tRf[(size_t)r * k + c] = (float)t;
   }
 }
 __global__ void k_hat_fwdR(int nr, int n, int k, const int* __restrict__ rverts, const int* __restrict__ btptr,
@@ -316,6 +301,7 @@ __device__ __forceinline__ void tri_gemv_body(int r, int lane, int n, bool lower
   const int c0 = lower ? 0 : r, c1 = lower ? r + 1 : n;
   const double* ar = A + (size_t)r * n;
   double s = 0.0;
+#pragma unroll 8
   for (int c = c0 + lane; c < c1; c += 32) s = fma(ar[c], x[c], s);
   s = hs_warp_sum(s);
   if (lane == 0) y[r] = s;
@@ -352,46 +338,60 @@ __global__ void k_tri_gemv32(int n, int lower, const float* __restrict__ A, cons
   tri_gemv32_body((blockIdx.x * blockDim.x + threadIdx.x) >> 5, threadIdx.x & 31, n, lower != 0, A, x, yf, yd);
 }
 
-// x_a = L_a^{-T}(y_a - F_a x_R); out[pverts[a] k + l] = scale x_a[l]; one warp per a
-__device__ __forceinline__ void bwdP_body(int a, int lane, int np, int k, const int* __restrict__ pverts,
+// x_a = L_a^{-T}(y_a - F_a x_R); out[pverts[a] k + l] = scale x_a[l].  One block of
+// HAT_THREADS per a: its warps share the k sums, lanes over the blocks; one warp
+// substitutes.
+__device__ __forceinline__ void bwdP_body(int a, int np, int k, const int* __restrict__ pverts,
                                           const int* __restrict__ bptr, const int* __restrict__ bcol,
                                           const double* __restrict__ F, const double* __restrict__ D,
                                           const double* __restrict__ yP, const double* __restrict__ xR,
                                           double scale, double* __restrict__ out) {
-  if (a >= np) return;
-  double acc[KMAX];
+  __shared__ double sz[KMAX];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int b0 = bptr[a], b1 = bptr[a + 1];
+  for (int i = w; i < k; i += HAT_THREADS / 32) {
+    double acc = 0.0;
+#pragma unroll 2
+    for (int bi = b0 + lane; bi < b1; bi += 32) {
+      const double* Fb = F + ((size_t)bi * k + i) * k;
+      const double* xr = xR + (size_t)bcol[bi] * k;
+      double f[KMAX], x[KMAX];
 #pragma unroll
-  for (int i = 0; i < KMAX; ++i) acc[i] = 0.0;
-  for (int bi = bptr[a] + lane; bi < bptr[a + 1]; bi += 32) {
-    const double* Fb = F + (size_t)bi * k * k;
-    const double* xr = xR + (size_t)bcol[bi] * k;
-    for (int c = 0; c < k; ++c) {
-      const double xc = xr[c];
+      for (int c = 0; c < KMAX; ++c)
+        if (c < k) {
+          f[c] = Fb[c];
+          x[c] = xr[c];
+        }
 #pragma unroll
-      for (int i = 0; i < KMAX; ++i)
-        if (i < k) acc[i] = fma(Fb[i * k + c], xc, acc[i]);
+      for (int c = 0; c < KMAX; ++c)
+        if (c < k) acc = fma(f[c], x[c], acc);
     }
+    acc = hs_warp_sum(acc);
+    if (lane == 0) sz[i] = yP[(size_t)a * k + i] - acc;
   }
-  double z[KMAX];
-#pragma unroll
-  for (int i = 0; i < KMAX; ++i) z[i] = (i < k) ? yP[(size_t)a * k + i] - hs_warp_sum(acc[i]) : 0.0;
-  if (lane != 0) return;
+  __syncthreads();
+  if (threadIdx.x != 0) return;
   const double* La = D + (size_t)a * k * k;
   const int v = pverts[a];
-  for (int i = k - 1; i >= 0; --i) {
-    double s = z[i];
-    for (int j = i + 1; j < k; ++j) s -= La[j * k + i] * z[j];
-    z[i] = s / La[i * k + i];
+  double z[KMAX];
+#pragma unroll
+  for (int i = KMAX - 1; i >= 0; --i) {
+    if (i >= k) continue;
+    double s = sz[i];
+#pragma unroll
+    for (int j = i + 1; j < KMAX; ++j)
+      if (j < k) s -= La[j * k + i] * z[j];
+    z[i] = div_rn(s, La[i * k + i]);
     out[(size_t)v * k + i] = scale * z[i];
   }
 }
-__global__ void k_hat_bwdP(int np, int n, int k, const int* __restrict__ pverts, const int* __restrict__ bptr,
-                           const int* __restrict__ bcol, const double* __restrict__ F, const double* __restrict__ D,
-                           const double* __restrict__ yP, const double* __restrict__ xR, double scale,
-                           double* __restrict__ out) {
-  (void)n;
-  bwdP_body((blockIdx.x * blockDim.x + threadIdx.x) >> 5, threadIdx.x & 31, np, k, pverts, bptr, bcol, F, D, yP, xR,
-            scale, out);
+__global__ void __launch_bounds__(HAT_THREADS) k_hat_bwdP(int np, int k, const int* __restrict__ pverts,
+                                                          const int* __restrict__ bptr, const int* __restrict__ bcol,
+                                                          const double* __restrict__ F, const double* __restrict__ D,
+                                                          const double* __restrict__ yP,
+                                                          const double* __restrict__ xR, double scale,
+                                                          double* __restrict__ out) {
+  bwdP_body(blockIdx.x, np, k, pverts, bptr, bcol, F, D, yP, xR, scale, out);
 }
 
 __device__ __forceinline__ void outR_body(int t, int nr, int k, const int* __restrict__ rverts,
@@ -585,10 +585,6 @@ __global__ void k_hat_bwdP_gen(int np, int k, const int* __restrict__ pverts, co
   if (!Dd.active) return;                                  \
   const int lb = blockIdx.x - off[inst];
 
-__global__ void kb_fwdP(const BDesc* __restrict__ desc, const int* __restrict__ off, int N) {
-  HS_BATCH_PROLOGUE
-  fwdP_body(lb * blockDim.x + threadIdx.x, Dd.np, Dd.n, Dd.k, Dd.pverts, Dd.D, Dd.uvec, Dd.yP);
-}
 __global__ void kb_fwdR(const BDesc* __restrict__ desc, const int* __restrict__ off, int N) {
   HS_BATCH_PROLOGUE
   fwdR_body((lb * blockDim.x + threadIdx.x) >> 5, threadIdx.x & 31, Dd.nr, Dd.n, Dd.k, Dd.rverts, Dd.btptr,
@@ -610,54 +606,34 @@ __global__ void kb_gemv_upper(const BDesc* __restrict__ desc, const int* __restr
   else
     tri_gemv_body((lb * blockDim.x + threadIdx.x) >> 5, threadIdx.x & 31, Dd.Rk, false, Dd.CinvT, Dd.v2, Dd.v1);
 }
-__global__ void kb_outR(const BDesc* __restrict__ desc, const int* __restrict__ off, int N) {
+// The last step of the core solve in one launch: the first blocks of a problem
+// scatter x_R (outR), the rest take a row of P each (bwdP); both only read x_R.
+__global__ void __launch_bounds__(HAT_THREADS) kb_out_bwd(const BDesc* __restrict__ desc, const int* __restrict__ off,
+                                                          int N) {
   HS_BATCH_PROLOGUE
-  outR_body(lb * blockDim.x + threadIdx.x, Dd.nr, Dd.k, Dd.rverts, Dd.v1, Dd.zscale, Dd.Bn);
-}
-// The last step of the core solve in one launch: the first ceil(Rk / 256)
-// blocks of a problem scatter x_R (outR), the rest substitute on the P rows
-// (bwdP); both only read x_R.
-__global__ void kb_out_bwd(const BDesc* __restrict__ desc, const int* __restrict__ off, int N) {
-  HS_BATCH_PROLOGUE
-  const int nout = (Dd.Rk + 255) / 256;
+  const int nout = (Dd.Rk + HAT_THREADS - 1) / HAT_THREADS;
   if (lb < nout) outR_body(lb * blockDim.x + threadIdx.x, Dd.nr, Dd.k, Dd.rverts, Dd.v1, Dd.zscale, Dd.Bn);
-  else
-    bwdP_body(((lb - nout) * blockDim.x + threadIdx.x) >> 5, threadIdx.x & 31, Dd.np, Dd.k, Dd.pverts, Dd.bptr,
-              Dd.bcol, Dd.F, Dd.D, Dd.yP, Dd.v1, Dd.zscale, Dd.Bn);
+  else if (lb - nout < Dd.np)
+    bwdP_body(lb - nout, Dd.np, Dd.k, Dd.pverts, Dd.bptr, Dd.bcol, Dd.F, Dd.D, Dd.yP, Dd.v1, Dd.zscale, Dd.Bn);
 }
-int batch_blocks_out_bwd(int Rk, int np) { return (int)(cdiv(Rk, 256) + cdiv((size_t)np * 32, 256)); }
-__global__ void kb_bwdP(const BDesc* __restrict__ desc, const int* __restrict__ off, int N) {
-  HS_BATCH_PROLOGUE
-  bwdP_body((lb * blockDim.x + threadIdx.x) >> 5, threadIdx.x & 31, Dd.np, Dd.k, Dd.pverts, Dd.bptr, Dd.bcol, Dd.F,
-            Dd.D, Dd.yP, Dd.v1, Dd.zscale, Dd.Bn);
-}
-int batch_blocks_fwdP(int np) { return (int)cdiv(np, 128); }
-int batch_blocks_warp_rows(int rows) { return (int)cdiv((size_t)rows * 32, 256); }
-int batch_blocks_outR(int Rk) { return (int)cdiv(Rk, 128); }
-void batch_launch_core_solve(cudaStream_t st, const BDesc* desc, int N, const int* off_fwdP, int nb_fwdP,
-                             const int* off_fwdR, int nb_fwdR, const int* off_gemv, int nb_gemv,
-                             const int* off_outR, int nb_outR, const int* off_bwdP, int nb_bwdP) {
+int batch_blocks_out_bwd(int Rk, int np) { return (int)cdiv(Rk, HAT_THREADS) + np; }
+int batch_blocks_warp_rows(int rows) { return (int)cdiv((size_t)rows * 32, HAT_THREADS); }
+void batch_launch_core_solve(cudaStream_t st, const BDesc* desc, int N, const int* off_fwdR, int nb_fwdR,
+                             const int* off_gemv, int nb_gemv, const int* off_out, int nb_out) {
   // a batch with no rows of a kind (e.g. no vertex outside the independent
   // set) launches nothing for it: a grid of zero blocks is not a launch
-  if (nb_fwdP > 0) {
-    count_launch();
-    kb_fwdP<<<nb_fwdP, 128, 0, st>>>(desc, off_fwdP, N);
-  }
   if (nb_fwdR > 0) {
     count_launch();
-    kb_fwdR<<<nb_fwdR, 256, 0, st>>>(desc, off_fwdR, N);
+    kb_fwdR<<<nb_fwdR, HAT_THREADS, 0, st>>>(desc, off_fwdR, N);
   }
   if (nb_gemv > 0) {
     count_launch(2);
-    kb_gemv_lower<<<nb_gemv, 256, 0, st>>>(desc, off_gemv, N);
-    kb_gemv_upper<<<nb_gemv, 256, 0, st>>>(desc, off_gemv, N);
+    kb_gemv_lower<<<nb_gemv, HAT_THREADS, 0, st>>>(desc, off_gemv, N);
+    kb_gemv_upper<<<nb_gemv, HAT_THREADS, 0, st>>>(desc, off_gemv, N);
   }
-  // off_outR / nb_outR: the merged out_bwd partition (batch_blocks_out_bwd)
-  (void)off_bwdP;
-  (void)nb_bwdP;
-  if (nb_outR > 0) {
+  if (nb_out > 0) {
     count_launch();
-    kb_out_bwd<<<nb_outR, 256, 0, st>>>(desc, off_outR, N);
+    kb_out_bwd<<<nb_out, HAT_THREADS, 0, st>>>(desc, off_out, N);
   }
 }
 
@@ -787,10 +763,9 @@ sdp_status schur_apply(sdp_problem* h, const double* u, double* out, double scal
   const bool lp = (prec != SDP_FP64) && Rk > 0;
   const bool gen = k > KMAX;
   if (lp) SDP_TRY(ensure_lowprec_core(h));
-  if (np > 0) {
+  if (np > 0 && gen) {
     count_launch();
-    if (gen) k_hat_fwdP_gen<<<cdiv(np, 128), 128, 0, st>>>(np, n, k, h->hs_pverts, h->hs_D, u, h->hs_yP);
-    else k_hat_fwdP<<<cdiv(np, 128), 128, 0, st>>>(np, n, k, h->hs_pverts, h->hs_D, u, h->hs_yP);
+    k_hat_fwdP_gen<<<cdiv(np, 128), 128, 0, st>>>(np, n, k, h->hs_pverts, h->hs_D, u, h->hs_yP);
   }
   if (Rk > 0) {
     count_launch();
@@ -799,17 +774,17 @@ sdp_status schur_apply(sdp_problem* h, const double* u, double* out, double scal
                                                                   h->hs_bp, h->hs_F, h->hs_yP, u, h->hs_v1,
                                                                   lp ? h->hs_v1f : nullptr);
     else
-      k_hat_fwdR<<<cdiv((size_t)nr * 32, 256), 256, 0, st>>>(nr, n, k, h->hs_rverts, h->hs_btptr, h->hs_btslot,
+      k_hat_fwdR<<<cdiv((size_t)Rk * 32, HAT_THREADS), HAT_THREADS, 0, st>>>(nr, n, k, h->hs_rverts, h->hs_btptr, h->hs_btslot,
                                                               h->hs_bp, h->hs_F, h->hs_yP, u, h->hs_v1,
                                                               lp ? h->hs_v1f : nullptr);
     // y_R = L_C^{-1} t_R and x_R = L_C^{-T} y_R (both inverses stored row-major)
     count_launch(2);
     if (lp) {
-      k_tri_gemv32<<<cdiv((size_t)Rk * 32, 256), 256, 0, st>>>(Rk, 1, h->hs_Cinv32, h->hs_v1f, h->hs_v2f, nullptr);
-      k_tri_gemv32<<<cdiv((size_t)Rk * 32, 256), 256, 0, st>>>(Rk, 0, h->hs_CinvT32, h->hs_v2f, nullptr, h->hs_v1);
+      k_tri_gemv32<<<cdiv((size_t)Rk * 32, HAT_THREADS), HAT_THREADS, 0, st>>>(Rk, 1, h->hs_Cinv32, h->hs_v1f, h->hs_v2f, nullptr);
+      k_tri_gemv32<<<cdiv((size_t)Rk * 32, HAT_THREADS), HAT_THREADS, 0, st>>>(Rk, 0, h->hs_CinvT32, h->hs_v2f, nullptr, h->hs_v1);
     } else {
-      k_tri_gemv<<<cdiv((size_t)Rk * 32, 256), 256, 0, st>>>(Rk, 1, h->hs_Cinv, h->hs_v1, h->hs_v2);
-      k_tri_gemv<<<cdiv((size_t)Rk * 32, 256), 256, 0, st>>>(Rk, 0, h->hs_CinvT, h->hs_v2, h->hs_v1);
+      k_tri_gemv<<<cdiv((size_t)Rk * 32, HAT_THREADS), HAT_THREADS, 0, st>>>(Rk, 1, h->hs_Cinv, h->hs_v1, h->hs_v2);
+      k_tri_gemv<<<cdiv((size_t)Rk * 32, HAT_THREADS), HAT_THREADS, 0, st>>>(Rk, 0, h->hs_CinvT, h->hs_v2, h->hs_v1);
     }
     count_launch();
     k_hat_outR<<<cdiv(Rk, 128), 128, 0, st>>>(nr, k, h->hs_rverts, h->hs_v1, scale, out);
@@ -822,8 +797,8 @@ sdp_status schur_apply(sdp_problem* h, const double* u, double* out, double scal
                                                                   h->hs_F, h->hs_D, h->hs_yP, xR, scale, out,
                                                                   h->hs_v3);
     else
-      k_hat_bwdP<<<cdiv((size_t)np * 32, 256), 256, 0, st>>>(np, n, k, h->hs_pverts, h->hs_bptr, h->hs_bcol,
-                                                              h->hs_F, h->hs_D, h->hs_yP, xR, scale, out);
+      k_hat_bwdP<<<np, HAT_THREADS, 0, st>>>(np, k, h->hs_pverts, h->hs_bptr, h->hs_bcol, h->hs_F, h->hs_D, h->hs_yP,
+                                             h->hs_v1, scale, out);
   }
   return SDP_OK;
 }

@@ -396,6 +396,10 @@ static sdp_status build(sdp_problem* h, int64_t nnzC, const int32_t* Ci, const i
   SDP_TRY(upload(h, &h->sptr, sptr));
   SDP_TRY(upload(h, &h->scon, scon));
   SDP_TRY(upload(h, &h->scoef, scoef));
+  h->single = (h->ncontrib == h->nnzV);
+  std::vector<double> sg(scoef.size());
+  for (size_t c = 0; c < scoef.size(); ++c) sg[c] = scoef[c] * ginv[scon[c]];
+  SDP_TRY(upload(h, &h->sg, sg));
   SDP_TRY(upload(h, &h->eptr, eptr));
   SDP_TRY(upload(h, &h->ep, ep));
   SDP_TRY(upload(h, &h->eq, eq));
@@ -413,6 +417,9 @@ static sdp_status build(sdp_problem* h, int64_t nnzC, const int32_t* Ci, const i
   SDP_TRY(upload(h, &h->kcra, kcra));
   SDP_TRY(upload(h, &h->kcrb, kcrb));
   SDP_TRY(upload(h, &h->hs_pverts, sp.pverts));
+  std::vector<int> pidx(n, -1);
+  for (size_t a = 0; a < sp.pverts.size(); ++a) pidx[sp.pverts[a]] = (int)a;
+  SDP_TRY(upload(h, &h->hs_pidx, pidx));
   SDP_TRY(upload(h, &h->hs_rverts, sp.rverts));
   SDP_TRY(upload(h, &h->hs_stype, sp.stype));
   SDP_TRY(upload(h, &h->hs_sa, sp.sa));
