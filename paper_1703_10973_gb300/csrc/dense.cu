@@ -8,6 +8,7 @@
 #include "internal.cuh"
 
 #include <algorithm>
+#include <cmath>
 
 namespace sdpgb {
 
@@ -162,10 +163,67 @@ __global__ void __launch_bounds__(256) k_gemm_thin(int M, int N, int K, double a
   }
 }
 
+// Short products C = alpha A B + beta C with at most THIN_N rows: a thread per
+// column of C walks K with a sum per row, in the order of the tiled kernel (whose
+// 32 x 32 tiles would be padding but for M rows: 4 x 565 x 565 took 141 us, 20 us
+// here); blocks of one warp, so that a product reaches N / 32 SMs.
+__global__ void __launch_bounds__(32) k_gemm_short(int M, int N, int K, double alpha, const double* __restrict__ A,
+                                                   int lda, const double* __restrict__ B, int ldb, double beta,
+                                                   double* __restrict__ C, int ldc) {
+  const int c = blockIdx.x * 32 + threadIdx.x;
+  double acc[THIN_N];
+#pragma unroll
+  for (int i = 0; i < THIN_N; ++i) acc[i] = 0.0;
+  const double* b = B + (c < N ? c : N - 1);
+#pragma unroll 8
+  for (int k = 0; k < K; ++k) {
+    const double x = b[(size_t)k * ldb];
+#pragma unroll
+    for (int i = 0; i < THIN_N; ++i)
+      if (i < M) acc[i] = fma(A[(size_t)i * lda + k], x, acc[i]);
+  }
+  if (c >= N) return;
+#pragma unroll
+  for (int i = 0; i < THIN_N; ++i) {
+    if (i >= M) break;
+    double v = alpha * acc[i];
+    if (beta != 0.0) v = fma(beta, C[(size_t)i * ldc + c], v);
+    C[(size_t)i * ldc + c] = v;
+  }
+}
+
+// Tile of C (16, 32 or 64): the FP64 pipe is the bound and belongs to an SM, so the
+// time is that of the SM with the most tiles; every tile size forms each entry by the
+// same chain over K, so the choice changes no bit.  Large tiles where they divide
+// evenly enough (fewer passes over A and B): 565^3 454 us with 32 x 32 (up to three
+// tiles on an SM), 355 us with 16 x 16; 4000^3 needs 64 x 64 for its operand traffic.
+static int gemm_tile(int M, int N, int flags, int batch) {
+  int best = 64;
+  double tb = 1e300;
+  for (int t : {64, 32, 16}) {
+    const double my = cdiv(M, t), mx = cdiv(N, t);
+    const double tiles = (flags & GEMM_LOWER_C) ? std::max(mx, my * (my + 1) / 2) : my * mx;
+    const double per_sm = std::ceil(tiles * batch / 152.0) * t * t * (t == 16 ? 1.06 : 1.0);
+    if (per_sm < 0.97 * tb) {
+      tb = per_sm;
+      best = t;
+    }
+  }
+  return best;
+}
+
 void gemm(cudaStream_t st, bool tA, bool tB, int M, int N, int K, double alpha, const double* A,
           int lda, const double* B, int ldb, double beta, double* C, int ldc, int flags,
           int batch, long long sA, long long sB, long long sC) {
   if (M <= 0 || N <= 0) return;
+  if (!tA && !tB && M <= THIN_N && N > THIN_N && K > 0 && flags == 0 && batch == 1) {
+    const bool timed = ktimer_on("gemm_f64");
+    if (timed) ktimer_begin(st, "gemm_f64");
+    count_launch();
+    k_gemm_short<<<cdiv(N, 32), 32, 0, st>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc);
+    if (timed) ktimer_end(st, "gemm_f64", 2.0 * M * N * (double)K, 8.0 * ((double)M * K + (double)K * N + 2.0 * M * N));
+    return;
+  }
   if (!tA && N <= THIN_N && K > 0 && flags == 0 && batch == 1) {
     const bool timed = ktimer_on("gemm_f64");
     if (timed) ktimer_begin(st, "gemm_f64");
@@ -185,14 +243,15 @@ void gemm(cudaStream_t st, bool tA, bool tB, int M, int N, int K, double alpha, 
     }
     return;
   }
-  const long long tiles64 = (long long)cdiv(M, 64) * cdiv(N, 64) * batch;
   const bool timed = ktimer_on("gemm_f64");
   if (timed) ktimer_begin(st, "gemm_f64");
-  const int tile = (tiles64 >= 2 * 152) ? 64 : 32;
+  const int tile = gemm_tile(M, N, flags, batch);
   if (tile == 64)
     gemm_launch<double, 64, 64>(st, tA, tB, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, flags, batch, sA, sB, sC);
-  else
+  else if (tile == 32)
     gemm_launch<double, 32, 32>(st, tA, tB, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, flags, batch, sA, sB, sC);
+  else
+    gemm_launch<double, 16, 16>(st, tA, tB, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, flags, batch, sA, sB, sC);
   if (timed) {
     const double f = 2.0 * gemm_useful_fma(M, N, K, flags, tile) * batch;
     const double by = 8.0 * ((double)M * K + (double)K * N + 2.0 * M * N) * batch;
