@@ -17,6 +17,7 @@ CASES = {
     "few": (lambda: si.mc_instance(3, 66, 1, 150, 3), (1, 4, 8)),
     "square": (lambda: si.mc_instance(33, 31, 1, 700, 4), (2, 5, 7, 9)),
     "many_neighbours": (lambda: si.mc_instance(150, 9, 1, 1200, 5), (1, 6, 8)),
+    "long_rows": (lambda: si.mc_instance(300, 320, 1, 1500, 6), (8,)),
     "general": (lambda: si.random_general(23, 40, 3, 2), (1, 3, 8)),
     "diag": (lambda: si.diag_constraint_instance(17, 1), (1, 2)),
 }
