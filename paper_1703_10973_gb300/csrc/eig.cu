@@ -704,9 +704,12 @@ __global__ void __launch_bounds__(SY_THREADS) k_sytrd_cluster_smem(int n, double
 // and read after barrier 2.  Every sum runs in a fixed order (those over the
 // reflector in 512 threads' order, p^T v in that of 16 warps), so the result does not
 // depend on timing.  An FP64 warp instruction holds its scheduler's pipe for 64
-// cycles: at n = 565 that bounds the first columns (14 us), latency the last ones.
-// With three barriers, 512 threads and the scalars on the way of the update a
-// column took 15.4 us on average (n = 565: 8.7 ms), now 12.0 us (6.8 ms).  At the end the rows are written back with
+// cycles however many lanes it serves, so the trees of the sums share instructions:
+// the first two levels in the warp that formed the sum, the others (and the 16 column
+// parts of a row) four lanes per row.  At n = 565 the pipe bounds the first columns,
+// latency the last ones.  With three barriers, 512 threads and the scalars on the way
+// of the update a column took 15.4 us on average (n = 565: 8.7 ms), with whole warps
+// for each sum 12.0 us (6.8 ms), now 10.9 us (6.1 ms).  At the end the rows are written back with
 // the lower part mirrored into the upper one: row j then holds the reflector in
 // A[j][j+1..], as the back-transformation expects.
 constexpr int SYL_THREADS = 1024;
@@ -723,11 +726,11 @@ __global__ void __launch_bounds__(SYL_THREADS, 1) k_sytrd_cluster_lower(int n, d
   // the vectors come first, at the same offset in every CTA (a remote access
   // maps the local offset); the packed rows, whose length depends on the
   // rank, follow them
-  double* p = sm + 3 * (size_t)n;   // n: tau A22 v (written remotely), then w
-  double* rowp = p + n;             // ceil(n / cs): row parts, then p_i, of the owned rows
+  double* p = sm + 3 * (size_t)n;   // n (at least 8): tau A22 v (written remotely), then w
+  double* rowp = p + max(n, 8);     // ceil(n / cs): row parts, then p_i, of the owned rows
   double* rows = rowp + (n + cs - 1) / cs;
   __shared__ double kpart[32];
-  __shared__ double red[32];
+  __shared__ double red[16][8];
   __shared__ double s_tau, s_beta, s_scale, s_K, s_w0;
   const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31, nw = SYL_THREADS / 32;
   for (int sl = 0; sl < slots; ++sl) {
@@ -744,19 +747,27 @@ __global__ void __launch_bounds__(SYL_THREADS, 1) k_sytrd_cluster_lower(int n, d
     if (i >= 2 && lane < cs) cluster.map_shared_rank(sm, lane)[n + i - 2] = ri[1];
   }
   cluster.sync();
-  // sum of squares of x[1..len) in the order of 512 threads: warps 0 to 15
+  // sum of squares of x[1..len) in the order of 512 threads: warps 0 to 15, whose sums
+  // (levels 4, 2, 1) end in scalars
   auto partial = [&](const double* x, int len) {
     if (tid < 512) {
       double s = 0.0;
-      for (int l = tid; l < len; l += 512)
-        if (l > 0) s = fma(x[l], x[l], s);
-      s = wsum(s);
-      if (lane == 0) red[wid] = s;
+      if (wid * 32 < len) {
+        for (int l = tid; l < len; l += 512)
+          if (l > 0) s = fma(x[l], x[l], s);
+        s += __shfl_xor_sync(0xffffffffu, s, 16);
+        s += __shfl_xor_sync(0xffffffffu, s, 8);
+      }
+      if (lane < 8) red[wid][lane] = s;
     }
   };
   auto scalars = [&](const double* x) {   // warp 0; the two quotients in two lanes
-    double s = (lane < 16) ? red[lane] : 0.0;
-    s = wsum(s);
+    // two lanes per warp of partial, four values each
+    const double* rd = red[lane >> 1] + (lane & 1);
+    double s = (rd[0] + rd[4]) + (rd[2] + rd[6]);
+    s += __shfl_xor_sync(0xffffffffu, s, 1);
+    s = __shfl_sync(0xffffffffu, s, (2 * lane) & 31);
+    s = wsum(lane < 16 ? s : 0.0);
     const double x0 = x[0];
     double tau = 0.0, beta = x0, scale = 0.0;
     if (s > 0.0) {
@@ -786,7 +797,8 @@ __global__ void __launch_bounds__(SYL_THREADS, 1) k_sytrd_cluster_lower(int n, d
     double* part = sm + (size_t)r2 * n;
     const double tau = s_tau, beta = s_beta;
     // ---- 1: column parts and row parts
-    for (int l = tid; l < len; l += SYL_THREADS) {
+    // (groups of four warps there and back: the first columns are the longest sums)
+    for (int l = (wid & 4) ? tid + 32 * (3 - 2 * (wid & 3)) : tid; l < len; l += SYL_THREADS) {
       const int c = j + 1 + l;
       int sl = (c >= rank) ? (c - rank) / cs + 1 : 0;   // first owned row > c
       double acc = 0.0;
@@ -812,20 +824,41 @@ __global__ void __launch_bounds__(SYL_THREADS, 1) k_sytrd_cluster_lower(int n, d
         a3 = fma(ri[l + 96], v[l + 96], a3);
       }
       for (; l < cnt; l += 32) a0 = fma(ri[l], v[l], a0);
-      const double rp = wsum((a0 + a1) + (a2 + a3));
-      if (lane == 0) rowp[sl] = rp;
+      double s = (a0 + a1) + (a2 + a3);
+      s += __shfl_xor_sync(0xffffffffu, s, 16);
+      s += __shfl_xor_sync(0xffffffffu, s, 8);
+      if (lane < 8) p[8 * (sl - sl0) + lane] = s;    // p is free until barrier 1
+    }
+    __syncthreads();
+    // the sums' levels 4, 2, 1, four lanes per row
+    for (int base = sl0 + 8 * wid; base < slots; base += 8 * nw) {
+      const int sl = base + (lane >> 2);
+      const double* x = p + 8 * (min(sl, slots - 1) - sl0) + (lane & 3);
+      double s = x[0] + x[4];
+      s += __shfl_xor_sync(0xffffffffu, s, 2);
+      s += __shfl_xor_sync(0xffffffffu, s, 1);
+      if ((lane & 3) == 0 && sl < slots) rowp[sl] = s;
     }
     cluster.sync();
     // ---- 2: p_i for the owned rows, broadcast
-    for (int sl = sl0 + wid; sl < slots; sl += nw) {
-      const int i = sl * cs + rank;
-      const int li = i - j - 1;
-      double x = (lane < cs) ? cluster.map_shared_rank(part, lane)[li] : 0.0;
-      x = wsum(x);
-      const double pi = (rowp[sl] + x) * tau;
-      if (lane < cs) cluster.map_shared_rank(p, lane)[li] = pi;
+    // four lanes per row, four of the 16 column parts and of the 16 copies each
+    for (int base = sl0 + 8 * wid; base < slots; base += 8 * nw) {
+      const int sl = base + (lane >> 2), q = lane & 3;
+      const bool on = sl < slots;
+      const int li = (on ? sl : slots - 1) * cs + rank - j - 1;
+      double x[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) x[u] = cluster.map_shared_rank(part, q + 4 * u)[li];
+      double s = (x[0] + x[2]) + (x[1] + x[3]);
+      s += __shfl_xor_sync(0xffffffffu, s, 2);
+      s += __shfl_xor_sync(0xffffffffu, s, 1);
+      const double pi = (rowp[on ? sl : slots - 1] + (s + 0.0)) * tau;   // a sum of zeros is +0
+      if (on) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) cluster.map_shared_rank(p, q + 4 * u)[li] = pi;
+      }
       __syncwarp();
-      if (lane == 0) rowp[sl] = pi;
+      if (on && q == 0) rowp[sl] = pi;
     }
     __syncthreads();
     if (wid == 0) {
@@ -919,7 +952,7 @@ static size_t sytrd_lower_smem_bytes(int n, int cs) {
     const int slots = (n - rank + cs - 1) / cs;
     most = std::max(most, (size_t)cs * slots * (slots - 1) / 2 + (size_t)slots * (rank + 1));
   }
-  return (4 * (size_t)n + (size_t)(n + cs - 1) / cs + most) * sizeof(double);
+  return (3 * (size_t)n + std::max(n, 8) + (size_t)(n + cs - 1) / cs + most) * sizeof(double);
 }
 
 // Cluster size of the shared-memory form for order n: 16 when the matrix and the
@@ -1049,11 +1082,9 @@ constexpr int SY_CLUSTER_MAX_N = 1024;
 
 // Order of preference: the one-triangle form in cluster shared memory
 // (n <= 880); the full-row form (n <= 656, where the device cannot run the
-// first); the L2-streaming cluster form; the cooperative grid form.  Alone, the
-// full-row form is as fast at n ~ 565 and faster for small n (two barriers per
-// column instead of three), but in a batch of concurrent problems the
-// one-triangle form's half-size shared-memory footprint leaves room on its 16
-// SMs for the other problems' kernels, which measured faster end to end.
+// first); the L2-streaming cluster form; above order 1024 the resident form, then the
+// cooperative grid form.  The one-triangle form also leaves more room on its 16 SMs
+// for the other problems' kernels of a batch.
 static sdp_status sytrd(cudaStream_t st, int n, double* A, EigWork* w) {
   if (n >= 3 && n <= SY_CLUSTER_MAX_N) {
     const int cs = sytrd_lower_cluster(n);
