@@ -535,83 +535,132 @@ void trmv_lower(cudaStream_t st, bool trans, int n, const double* L, int ldl, co
 // ---------------------------------------------------------------------------
 constexpr int NB = 64;
 
-// Factor the nbs x nbs (nbs <= BS) diagonal block in place (lower).  256
-// threads; thread t keeps the BS^2 / 256 entries (i, l) with l = t % BS and
-// i = t / BS + (256 / BS) s in registers.  Per column j: the owner of (j, j)
-// forms the pivot, the owners of column j scale it and publish it to shared
-// memory, and every thread applies the rank-1 update to its entries -- two
-// barriers per column and one reciprocal instead of a division per entry.  The
-// published column alternates between two buffers, so the writers of column
-// j + 1 never overwrite a value that a thread still finishing step j reads.
-// FP64 issue slots are the scarce resource on this GPU (a warp instruction
-// costs the same with most lanes masked), so the factorisation uses 32 x 32
-// diagonal blocks: the per-column work of every thread stays at 4 entries.
-template <int BS>
-__global__ void __launch_bounds__(256) k_potrf_diag(int nbs, double* A, int lda, int* info, int base,
-                                                    double floor_) {
-  constexpr int RS = 256 / BS;        // row stride of a thread's entries
-  constexpr int PER = BS / RS;        // entries per thread
-  __shared__ double colbuf[2][BS];
-  __shared__ double s_rinv;
-  const int t = threadIdx.x;
-  const int l = t % BS, i0 = t / BS;
-  double a[PER];
-#pragma unroll
-  for (int s = 0; s < PER; ++s) {
-    const int i = i0 + RS * s;
-    a[s] = (i < nbs && l < nbs && l <= i) ? A[(size_t)i * lda + l] : 0.0;
-  }
-  for (int j = 0; j < nbs; ++j) {
-    double* colj = colbuf[j & 1];
-    if (l == j) {
-#pragma unroll
-      for (int s = 0; s < PER; ++s) {
-        if (i0 + RS * s != j) continue;
-        double p = a[s];
-        if (floor_ > 0.0) {
-          // the matrix is known to satisfy A >= floor I, so every Cholesky pivot
-          // (a Schur-complement diagonal) is >= floor; smaller ones are rounding
-          if (!(p >= floor_)) {
-            if (info) atomicAdd(info + 1, 1);
-            p = floor_;
-          }
-        } else if (!(p > 0.0)) {
-          if (info && *info == 0) *info = base + j + 1;
-          p = 1.0;
-        }
-        const double dj = sqrt(p);
-        a[s] = dj;
-        colj[j] = dj;
-        s_rinv = 1.0 / dj;
+// Factor the nbs x nbs (nbs <= PB) diagonal block held in a (lower) and store it.  Four
+// warps, one per scheduler (FP64 issue slots are the scarce resource: a warp
+// instruction holds its scheduler's pipe for 64 cycles however many lanes it serves);
+// lane i keeps row i, warp w the columns w, w + 4, ... in registers.  Per column j the
+// warp that owns it takes the pivot's root and its reciprocal, scales the column and
+// publishes it; after the barrier every warp updates its columns, the owner of j + 1
+// that column first, and goes on to its pivot while the others update.  So a column
+// costs the chain update, root, reciprocal, scaling, one instruction each but for the
+// root and the reciprocal.  The published column alternates between two buffers.
+// 36 us per block; 256 threads with two barriers a column and eight warps scaling
+// each column took 48 us.
+constexpr int PB = 32;
+constexpr int PB_THREADS = 128;
+__device__ __forceinline__ void potrf_diag_body(int nbs, double (&a)[PB / 4], double (&col)[2][PB], double* A, int lda,
+                                                int* info, int base, double floor_, double* rcp) {
+  const int i = threadIdx.x & 31, w = threadIdx.x >> 5;
+  auto pivot = [&](int j, double& x) {   // x: the owner's entries of column j
+    double p = __shfl_sync(0xffffffffu, x, j);
+    if (floor_ > 0.0) {
+      // the matrix is known to satisfy A >= floor I, so every Cholesky pivot
+      // (a Schur-complement diagonal) is >= floor; smaller ones are rounding
+      if (!(p >= floor_)) {
+        if (info && i == 0) atomicAdd(info + 1, 1);
+        p = floor_;
       }
+    } else if (!(p > 0.0)) {
+      if (info && i == 0 && *info == 0) *info = base + j + 1;
+      p = 1.0;
+    }
+    const double dj = sqrt(p);
+    const double r = 1.0 / dj;
+    if (i == j) rcp[j] = r;               // for the panel's solve
+    x = (i == j) ? dj : x * r;            // rows above the diagonal hold garbage, never read
+    col[j & 1][i] = x;
+  };
+  if (w == 0) pivot(0, a[0]);
+#pragma unroll
+  for (int j = 0; j < PB; ++j) {
+    if (j >= nbs) break;
+    __syncthreads();
+    const double* cj = col[j & 1];
+    const double ci = cj[i];
+    const bool next = (j + 1 < PB) && w == ((j + 1) & 3) && j + 1 < nbs;
+    if (next) {
+      const int c = (j + 1) >> 2;
+      a[c < PB / 4 ? c : 0] = fma(-ci, cj[(j + 1) & 31], a[c < PB / 4 ? c : 0]);
+      pivot(j + 1, a[c < PB / 4 ? c : 0]);
+    }
+#pragma unroll
+    for (int c = 0; c < PB / 4; ++c) {
+      const int l = w + 4 * c;
+      if (l > j + (next ? 1 : 0)) a[c] = fma(-ci, cj[l], a[c]);
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < PB / 4; ++c) {
+    const int l = w + 4 * c;
+    if (i < nbs && l < nbs) A[(size_t)i * lda + l] = (l <= i) ? a[c] : 0.0;
+  }
+}
+__global__ void __launch_bounds__(PB_THREADS) k_potrf_diag(int nbs, double* A, int lda, int* info, int base,
+                                                           double floor_, double* rcp) {
+  __shared__ double col[2][PB];
+  const int i = threadIdx.x & 31, w = threadIdx.x >> 5;
+  double a[PB / 4];
+#pragma unroll
+  for (int c = 0; c < PB / 4; ++c) {
+    const int l = w + 4 * c;
+    a[c] = (i < nbs && l <= i) ? A[(size_t)i * lda + l] : 0.0;
+  }
+  potrf_diag_body(nbs, a, col, A, lda, info, base, floor_, rcp);
+}
+
+// Trailing update C -= P P^T (lower 32 x 32 tiles, P: rows x PB) and, in block 0, the
+// factorisation of the next diagonal block, C's first tile: that serial chain runs
+// beside the update instead of behind it (and is no launch of its own).  Sums in the
+// order of the tiled product, k from 0.
+__global__ void __launch_bounds__(PB_THREADS) k_potrf_update(int rows, const double* P, double* C, int lda, int* info,
+                                                             int base, double floor_, double* rcp) {
+  __shared__ double As[PB][PB + 1], Bs[PB][PB + 1], col[2][PB];
+  int ti = (int)((sqrtf(8.0f * (float)blockIdx.x + 1.0f) - 1.0f) * 0.5f);   // lower tile number blockIdx.x
+  while ((ti + 1) * (ti + 2) / 2 <= (int)blockIdx.x) ++ti;
+  while (ti * (ti + 1) / 2 > (int)blockIdx.x) --ti;
+  const int tj = (int)blockIdx.x - ti * (ti + 1) / 2;
+  const int bm = ti * PB, bn = tj * PB;
+#pragma unroll
+  for (int t = threadIdx.x; t < PB * PB; t += PB_THREADS) {
+    const int r = t / PB, k = t % PB;
+    As[k][r] = (bm + r < rows) ? P[(size_t)(bm + r) * lda + k] : 0.0;
+    Bs[k][r] = (bn + r < rows) ? P[(size_t)(bn + r) * lda + k] : 0.0;
+  }
+  if (blockIdx.x == 0) {
+    const int i = threadIdx.x & 31, w = threadIdx.x >> 5, nbs = min(PB, rows);
+    double a[PB / 4], acc[PB / 4];
+#pragma unroll
+    for (int c = 0; c < PB / 4; ++c) {
+      const int l = w + 4 * c;
+      a[c] = (i < nbs && l <= i) ? C[(size_t)i * lda + l] : 0.0;
+      acc[c] = 0.0;
     }
     __syncthreads();
-    if (l == j) {
-      const double r = s_rinv;
+#pragma unroll 4
+    for (int k = 0; k < PB; ++k)
 #pragma unroll
-      for (int s = 0; s < PER; ++s) {
-        const int i = i0 + RS * s;
-        if (i > j && i < nbs) {
-          a[s] *= r;
-          colj[i] = a[s];
-        }
-      }
-    }
-    __syncthreads();
-    if (l > j && l < nbs) {
-      const double cl = colj[l];
+      for (int c = 0; c < PB / 4; ++c) acc[c] = fma(As[k][i], As[k][w + 4 * c], acc[c]);
 #pragma unroll
-      for (int s = 0; s < PER; ++s) {
-        const int i = i0 + RS * s;
-        if (i >= l && i < nbs) a[s] = fma(-colj[i], cl, a[s]);
-      }
-    }
+    for (int c = 0; c < PB / 4; ++c) a[c] = a[c] - acc[c];
+    potrf_diag_body(nbs, a, col, C, lda, info, base, floor_, rcp);
+    return;
   }
+  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;   // rows ty + 8 u, columns tx + 16 v
+  double acc[4][2] = {};
+  __syncthreads();
+#pragma unroll 4
+  for (int k = 0; k < PB; ++k)
 #pragma unroll
-  for (int s = 0; s < PER; ++s) {
-    const int i = i0 + RS * s;
-    if (i < nbs && l < nbs) A[(size_t)i * lda + l] = (l <= i) ? a[s] : 0.0;
-  }
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int v = 0; v < 2; ++v) acc[u][v] = fma(As[k][ty + 8 * u], Bs[k][tx + 16 * v], acc[u][v]);
+#pragma unroll
+  for (int u = 0; u < 4; ++u)
+#pragma unroll
+    for (int v = 0; v < 2; ++v) {
+      const int r = bm + ty + 8 * u, c = bn + tx + 16 * v;
+      if (r < rows && c < rows) C[(size_t)r * lda + c] -= acc[u][v];
+    }
 }
 
 // Triangular solves with one kbs x kbs (kbs <= 64) diagonal block of L, one warp
@@ -621,46 +670,57 @@ __global__ void __launch_bounds__(256) k_potrf_diag(int nbs, double* A, int lda,
 // updated (no division: the reciprocals of the diagonal are precomputed).
 //   trans = false:  L x = b  (forward);   trans = true:  L^T x = b  (backward)
 // The right solve X L^T = P of the Cholesky panel is the forward solve on each
-// row of P.
+// row of P, with the reciprocals from the factorisation (rcp).
+// KB = 32 (the Cholesky panel: one entry per lane) or 64; the vector's loads are on
+// their way while L is staged.
 constexpr int TRSV_WARPS = 4;
+template <int KB>
 __global__ void __launch_bounds__(32 * TRSV_WARPS) k_trsv_warp(int kbs, bool trans, const double* __restrict__ L,
                                                                int ldl, double* __restrict__ X, int nvec,
-                                                               int vstride, int estride) {
-  __shared__ double sl[NB][NB + 1];
-  __shared__ double rd[NB];
-  for (int t = threadIdx.x; t < kbs * kbs; t += blockDim.x) {
-    const int i = t / kbs, j = t % kbs;
-    sl[i][j] = (j <= i) ? L[(size_t)i * ldl + j] : 0.0;
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < kbs; i += blockDim.x) rd[i] = 1.0 / sl[i][i];
-  __syncthreads();
+                                                               int vstride, int estride, const double* rcp) {
+  __shared__ double sl[KB][KB + 1];
+  __shared__ double rd[KB];
   const int lane = threadIdx.x & 31;
   const int v = blockIdx.x * TRSV_WARPS + (threadIdx.x >> 5);
-  if (v >= nvec) return;
-  double* x = X + (size_t)v * vstride;
+  double* x = X + (size_t)(v < nvec ? v : 0) * vstride;
   const int e0 = lane, e1 = lane + 32;
   double x0 = (e0 < kbs) ? x[(size_t)e0 * estride] : 0.0;
-  double x1 = (e1 < kbs) ? x[(size_t)e1 * estride] : 0.0;
+  double x1 = (KB > 32 && e1 < kbs) ? x[(size_t)e1 * estride] : 0.0;
+#pragma unroll 4
+  for (int t = threadIdx.x; t < KB * KB; t += 32 * TRSV_WARPS) {
+    const int i = t / KB, j = t % KB;
+    sl[i][j] = (i < kbs && j <= i) ? L[(size_t)i * ldl + j] : 0.0;
+  }
+  if (rcp && (int)threadIdx.x < kbs) rd[threadIdx.x] = rcp[threadIdx.x];
+  __syncthreads();
+  if (!rcp) {
+    if ((int)threadIdx.x < kbs) rd[threadIdx.x] = 1.0 / sl[threadIdx.x][threadIdx.x];
+    __syncthreads();
+  }
+  if (v >= nvec) return;
   if (!trans) {
     for (int j = 0; j < kbs; ++j) {
-      const double xj = __shfl_sync(0xffffffffu, (j < 32) ? x0 : x1, j & 31) * rd[j];
+      const double xj = __shfl_sync(0xffffffffu, (KB == 32 || j < 32) ? x0 : x1, j & 31) * rd[j];
       if (e0 == j) x0 = xj;
-      if (e1 == j) x1 = xj;
       if (e0 > j && e0 < kbs) x0 = fma(-sl[e0][j], xj, x0);
-      if (e1 > j && e1 < kbs) x1 = fma(-sl[e1][j], xj, x1);
+      if (KB > 32) {
+        if (e1 == j) x1 = xj;
+        if (e1 > j && e1 < kbs) x1 = fma(-sl[e1 < KB ? e1 : 0][j], xj, x1);
+      }
     }
   } else {
     for (int j = kbs - 1; j >= 0; --j) {
-      const double xj = __shfl_sync(0xffffffffu, (j < 32) ? x0 : x1, j & 31) * rd[j];
+      const double xj = __shfl_sync(0xffffffffu, (KB == 32 || j < 32) ? x0 : x1, j & 31) * rd[j];
       if (e0 == j) x0 = xj;
-      if (e1 == j) x1 = xj;
       if (e0 < j) x0 = fma(-sl[j][e0], xj, x0);
-      if (e1 < j) x1 = fma(-sl[j][e1], xj, x1);
+      if (KB > 32) {
+        if (e1 == j) x1 = xj;
+        if (e1 < j) x1 = fma(-sl[j][e1 < KB ? e1 : 0], xj, x1);
+      }
     }
   }
   if (e0 < kbs) x[(size_t)e0 * estride] = x0;
-  if (e1 < kbs) x[(size_t)e1 * estride] = x1;
+  if (KB > 32 && e1 < kbs) x[(size_t)e1 * estride] = x1;
 }
 
 size_t potrf_work_doubles(int n) { return (size_t)NB * NB + (size_t)n * NB; }
@@ -673,24 +733,19 @@ void potrf(cudaStream_t st, int n, double* A, int lda, int* info_dev, double* wo
 // floor are raised to floor and counted in info_dev[1] instead of failing.
 void potrf_floor(cudaStream_t st, int n, double* A, int lda, int* info_dev, double* work, double floor_) {
 
-  (void)work;
   ktimer_begin(st, "potrf");
   cudaMemsetAsync(info_dev, 0, 2 * sizeof(int), st);
-  constexpr int PB = 32;   // diagonal block of the factorisation (see k_potrf_diag)
-  for (int k0 = 0; k0 < n; k0 += PB) {
-    const int kbs = std::min(PB, n - k0);
+  count_launch();
+  k_potrf_diag<<<1, PB_THREADS, 0, st>>>(std::min(PB, n), A, lda, info_dev, 0, floor_, work);
+  for (int k0 = 0; k0 + PB < n; k0 += PB) {
     double* Akk = A + (size_t)k0 * lda + k0;
-    count_launch();
-    k_potrf_diag<PB><<<1, 256, 0, st>>>(kbs, Akk, lda, info_dev, k0, floor_);
-    const int r0 = k0 + kbs;
-    const int rows = n - r0;
-    if (rows <= 0) break;
+    const int r0 = k0 + PB, rows = n - r0, tiles = (int)cdiv(rows, PB);
     double* P = A + (size_t)r0 * lda + k0;
     // panel: P <- P L_kk^{-T}, a forward solve on each row (one warp per row)
-    count_launch();
-    k_trsv_warp<<<cdiv(rows, TRSV_WARPS), 32 * TRSV_WARPS, 0, st>>>(kbs, false, Akk, lda, P, rows, lda, 1);
-    // trailing: A22 -= P P^T (lower tiles only)
-    gemm(st, false, true, rows, rows, kbs, -1.0, P, lda, P, lda, 1.0, A + (size_t)r0 * lda + r0, lda, 1);
+    count_launch(2);
+    k_trsv_warp<PB><<<cdiv(rows, TRSV_WARPS), 32 * TRSV_WARPS, 0, st>>>(PB, false, Akk, lda, P, rows, lda, 1, work);
+    k_potrf_update<<<tiles * (tiles + 1) / 2, PB_THREADS, 0, st>>>(rows, P, A + (size_t)r0 * lda + r0, lda, info_dev, r0,
+                                                                   floor_, work);
   }
   zero_upper(st, n, A, lda);
   ktimer_end(st, "potrf", (double)n * n * n / 3.0, 8.0 * n * n);
@@ -720,8 +775,8 @@ void trsm_left_lower_ex(cudaStream_t st, bool trans, int n, int nrhs, const doub
       const int nc = lower_rhs ? std::min(nrhs, k0 + kbs) : nrhs;
       double* Bk = B + (size_t)k0 * ldb;
       count_launch();
-      k_trsv_warp<<<cdiv(nc, TRSV_WARPS), 32 * TRSV_WARPS, 0, st>>>(kbs, false, L + (size_t)k0 * ldl + k0, ldl, Bk, nc,
-                                                                    1, ldb);
+      k_trsv_warp<NB><<<cdiv(nc, TRSV_WARPS), 32 * TRSV_WARPS, 0, st>>>(kbs, false, L + (size_t)k0 * ldl + k0, ldl, Bk, nc,
+                                                                    1, ldb, nullptr);
       const int r0 = k0 + kbs;
       if (r0 < n)
         gemm(st, false, false, n - r0, nc, kbs, -1.0, L + (size_t)r0 * ldl + k0, ldl, Bk, ldb, 1.0,
@@ -732,8 +787,8 @@ void trsm_left_lower_ex(cudaStream_t st, bool trans, int n, int nrhs, const doub
       const int k0 = b * NB, kbs = std::min(NB, n - k0);
       double* Bk = B + (size_t)k0 * ldb;
       count_launch();
-      k_trsv_warp<<<cdiv(nrhs, TRSV_WARPS), 32 * TRSV_WARPS, 0, st>>>(kbs, true, L + (size_t)k0 * ldl + k0, ldl, Bk,
-                                                                      nrhs, 1, ldb);
+      k_trsv_warp<NB><<<cdiv(nrhs, TRSV_WARPS), 32 * TRSV_WARPS, 0, st>>>(kbs, true, L + (size_t)k0 * ldl + k0, ldl, Bk,
+                                                                      nrhs, 1, ldb, nullptr);
       if (k0 > 0)
         gemm(st, true, false, k0, nrhs, kbs, -1.0, L + (size_t)k0 * ldl, ldl, Bk, ldb, 1.0, B, ldb);
     }
