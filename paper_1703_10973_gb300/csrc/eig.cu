@@ -1351,152 +1351,97 @@ __device__ __forceinline__ double hash_unif(unsigned long long x) {
   return (double)(x >> 11) * (2.0 / 9007199254740992.0) - 1.0;  // [-1, 1)
 }
 
-// One eigenvector per thread.  With blocks == nullptr the whole tridiagonal is
-// used; otherwise thread t works on the unreduced diagonal block that owns the
-// eigenvalue (src[t] is its row, blocks = {blockid, bstart, bend}) and the
-// vector is zero outside that block.
-__global__ void k_stein(int nfull, const double* __restrict__ dfull, const double* __restrict__ efull,
-                        const double* __restrict__ wsel, int cnt, double* __restrict__ ws, int bstride,
-                        double* __restrict__ Eout, int ldE, int tbase, const int* __restrict__ src,
-                        const int* __restrict__ blocks) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= cnt) return;
-  int s0 = 0, s1 = nfull;
-  if (blocks) {
-    const int b = blocks[src[t]];
-    s0 = blocks[nfull + b];
-    s1 = blocks[2 * nfull + b];
-  }
-  const int n = s1 - s0;
-  const double* d = dfull + s0;
-  const double* e = efull + s0;
-#define WS(f, i) ws[((size_t)(f) * nfull + (i)) * bstride + t]
-  const double lam = wsel[t];
-  double tnorm = 0.0;
-  for (int i = 0; i < n; ++i) {
-    const double r = fabs(d[i]) + (i > 0 ? fabs(e[i - 1]) : 0.0) + (i + 1 < n ? fabs(e[i]) : 0.0);
-    tnorm = fmax(tnorm, r);
-  }
-  const double tol = fmax(DBL_EPSILON * tnorm, DBL_MIN);
-  // fields: 0 a (diag of U), 1 b (super), 2 c (multipliers), 3 d2 (second super), 4 y, 5 pivot flag
-  for (int i = 0; i < n; ++i) {
-    WS(0, i) = d[i] - lam;
-    WS(1, i) = (i + 1 < n) ? e[i] : 0.0;
-    WS(2, i) = (i + 1 < n) ? e[i] : 0.0;
-    WS(3, i) = 0.0;
-    WS(5, i) = 0.0;
-  }
-  for (int k = 0; k + 1 < n; ++k) {
-    const double ak = WS(0, k), bk = WS(1, k), ck = WS(2, k);
-    const double ak1 = WS(0, k + 1);
-    const double bk1 = (k + 2 < n) ? WS(1, k + 1) : 0.0;
+// Elimination with partial pivoting of V vectors by one warp, four lanes each.
+template <int V>
+__device__ __forceinline__ void stein_eliminate(int lane, int nmax, const int* sh_s0, const int* sh_n, const double* sh_lam,
+                                                const double* __restrict__ dfull, const double* __restrict__ efull,
+                                                double* fa, double* fb, double* fc, double* fd, unsigned char* ff) {
+  const int v = (lane >> 2) % V, sub = lane & 3;   // lanes past 4 V repeat the first vectors, unstored
+  const bool mine = lane < 4 * V && sub == 0;
+  const int n = sh_n[v];
+  const double* d = dfull + sh_s0[v];
+  const double* e = efull + sh_s0[v];
+  const double lam = sh_lam[v];
+  double ak = (n > 0) ? d[0] - lam : 1.0;
+  double bk = (n > 1) ? e[0] : 0.0;
+  double ck = bk, dn = (n > 1) ? d[1] : 0.0, en = (n > 2) ? e[1] : 0.0;
+  for (int k = 0; k + 1 < nmax; ++k) {
+    const bool on = k + 1 < n;
+    const double ak1 = dn - lam;
+    const double bk1 = en;                               // 0 from row n - 2 on
+    const double ckn = en;
+    dn = (k + 2 < n) ? d[k + 2] : 0.0;                   // next step's entries on their way
+    en = (k + 3 < n) ? e[k + 2] : 0.0;
     const double scale1 = fabs(ak) + fabs(bk);
     const double scale2 = fabs(ck) + fabs(ak1) + fabs(bk1);
-    const double piv1 = (scale1 == 0.0) ? 0.0 : fabs(ak) / scale1;
-    if (ck == 0.0) {
-      WS(5, k) = 0.0;
-      WS(3, k) = 0.0;
-    } else {
-      const double piv2 = fabs(ck) / scale2;
-      if (piv2 <= piv1) {
-        const double mult = ck / ak;
-        WS(5, k) = 0.0;
-        WS(2, k) = mult;
-        WS(0, k + 1) = ak1 - mult * bk;
-        WS(3, k) = 0.0;
+    const double num = (sub == 0) ? fabs(ak) : (sub == 1) ? fabs(ck) : (sub == 2) ? ck : ak;
+    const double den = (sub == 0) ? scale1 : (sub == 1) ? scale2 : (sub == 2) ? ak : ck;
+    const double q = num / den;
+    const int b4 = lane & ~3;
+    const double q0 = __shfl_sync(0xffffffffu, q, b4), piv2 = __shfl_sync(0xffffffffu, q, b4 + 1);
+    const double q2 = __shfl_sync(0xffffffffu, q, b4 + 2), q3 = __shfl_sync(0xffffffffu, q, b4 + 3);
+    const double piv1 = (scale1 == 0.0) ? 0.0 : q0;
+    if (on) {
+      double oa = ak, ob = bk, oc = 0.0, od = 0.0, na, nb = bk1;
+      unsigned char fl = 0;
+      if (ck == 0.0) {
+        na = ak1;
+      } else if (piv2 <= piv1) {
+        oc = q2;
+        na = ak1 - q2 * bk;
       } else {
-        const double mult = ak / ck;
-        WS(5, k) = 1.0;
-        WS(0, k) = ck;
-        WS(0, k + 1) = bk - mult * ak1;
+        fl = 1;
+        oa = ck;
+        ob = ak1;
+        oc = q3;
+        na = bk - q3 * ak1;
         if (k + 2 < n) {
-          WS(3, k) = bk1;
-          WS(1, k + 1) = -mult * bk1;
+          od = bk1;
+          nb = -q3 * bk1;
         } else {
-          WS(3, k) = 0.0;
+          nb = 0.0;
         }
-        WS(1, k) = ak1;
-        WS(2, k) = mult;
       }
+      if (mine) {
+        const size_t x = (size_t)k * V + v;
+        fa[x] = oa;
+        fb[x] = ob;
+        fc[x] = oc;
+        fd[x] = od;
+        ff[x] = fl;
+      }
+      ak = na;
+      bk = nb;
+      ck = ckn;
     }
   }
-  // reciprocal pivots (tiny pivots replaced by +-tol) so the solves only multiply
-  for (int k = 0; k < n; ++k) {
-    double ak = WS(0, k);
-    if (fabs(ak) < tol) ak = (ak >= 0.0) ? tol : -tol;
-    WS(0, k) = 1.0 / ak;
-  }
-  for (int i = 0; i < n; ++i) WS(4, i) = hash_unif(((unsigned long long)(tbase + t) << 32) ^ (unsigned long long)i);
-  for (int iter = 0; iter < 3; ++iter) {
-    // forward: P L^{-1}
-    for (int k = 1; k < n; ++k) {
-      if (WS(5, k - 1) == 0.0) {
-        WS(4, k) = WS(4, k) - WS(2, k - 1) * WS(4, k - 1);
-      } else {
-        const double tmp = WS(4, k - 1);
-        const double yk = WS(4, k);
-        WS(4, k - 1) = yk;
-        WS(4, k) = tmp - WS(2, k - 1) * yk;
-      }
-    }
-    // backward: U^{-1} with tiny pivots replaced by +-tol.  Each tiny pivot
-    // multiplies by up to 1/tol, so a cluster of them can overflow: whenever an
-    // entry passes 2^400 the whole vector (solved part and remaining
-    // right-hand side alike) is scaled by 2^-400, which keeps the system
-    // consistent; the vector is normalised afterwards anyway.
-    double ymax = 0.0;
-    for (int k = n - 1; k >= 0; --k) {
-      double tmp = WS(4, k);
-      if (k + 1 < n) tmp -= WS(1, k) * WS(4, k + 1);
-      if (k + 2 < n) tmp -= WS(3, k) * WS(4, k + 2);
-      double yk = tmp * WS(0, k);
-      if (!(fabs(yk) < 0x1p+400)) {
-        for (int j = 0; j < n; ++j) WS(4, j) *= 0x1p-400;
-        ymax *= 0x1p-400;
-        yk = (tmp * 0x1p-400) * WS(0, k);
-      }
-      WS(4, k) = yk;
-      ymax = fmax(ymax, fabs(yk));
-    }
-    // normalise (scale by the max first to avoid overflow)
-    const double inv = (ymax > 0.0) ? 1.0 / ymax : 1.0;
-    double nrm = 0.0;
-    for (int k = 0; k < n; ++k) {
-      const double yk = WS(4, k) * inv;
-      WS(4, k) = yk;
-      nrm = fma(yk, yk, nrm);
-    }
-    const double sc = 1.0 / sqrt(nrm);
-    for (int k = 0; k < n; ++k) WS(4, k) *= sc;
-  }
-  double* out = Eout + (size_t)t * ldE;
-  for (int k = 0; k < s0; ++k) out[k] = 0.0;
-  for (int k = 0; k < n; ++k) out[s0 + k] = WS(4, k);
-  for (int k = s1; k < nfull; ++k) out[k] = 0.0;
-#undef WS
+  if (mine && n > 0) fa[(size_t)(n - 1) * V + v] = ak;
 }
 
-// The same inverse iteration with the working arrays in shared memory: a block of
-// 128 threads takes V vectors; what runs along the tridiagonal (elimination,
-// substitutions, the sum of squares) runs in lanes of warp 0, everything
-// elementwise in all threads.  Every operation and its order are those of k_stein,
-// so the vectors are the same bit for bit.  The elimination's pivot test needs two
+// Inverse iteration, three solves per vector.  With blocks == nullptr the whole
+// tridiagonal is used; otherwise a vector works on the unreduced diagonal block that
+// owns its eigenvalue (src[t] is its row, blocks = {blockid, bstart, bend}) and is zero
+// outside that block.  A block of 128 threads takes V vectors; what runs along the
+// tridiagonal (elimination, substitutions, the sum of squares) runs in lanes of warp
+// 0, everything elementwise in all threads.  The elimination's pivot test needs two
 // quotients and its multiplier a third: four lanes per vector compute |a|/(|a|+|b|),
 // |c|/(|c|+|a'|+|b'|), c/a and a/c side by side and take what the test selects.
 // Bound by that serial chain of FP64 instructions (64 cycles of a scheduler's pipe
-// each); k_stein walks the same chain through L2.  n = 565: 4.2 ms -> 1.3 ms for all
-// vectors, 1.0 ms for four; n = 2000, one vector: 19 ms -> 3.5 ms.
+// each).  Two forms with the same operations in the same order, for the working arrays
+// in shared memory and in global memory; a thread per vector through L2 took 4.2 ms at
+// n = 565, 22.8 ms at n = 2000 for all vectors, here 1.1 and 4.1 ms.
 // Fields, index k, vector v at [(f n + k) V + v]: 0 a (reciprocal pivots), 1 b,
 // 2 c (multipliers), 3 d2, 4 y; then n V pivot flags.
 constexpr int STEIN_THREADS = 128;
-static size_t stein_sm_bytes(int n, int V) { return (size_t)n * V * (5 * sizeof(double) + 1) + 16; }
-template <int V>
+constexpr int STEIN_GL_V = 8;   // vectors per block in global memory, one in shared memory
+static size_t stein_sm_bytes(int n) { return (size_t)n * (5 * sizeof(double) + 1) + 16; }
 __global__ void __launch_bounds__(STEIN_THREADS) k_stein_sm(int nfull, const double* __restrict__ dfull,
                                                             const double* __restrict__ efull,
                                                             const double* __restrict__ wsel, int cnt,
                                                             double* __restrict__ Eout, int ldE, int tbase,
                                                             const int* __restrict__ src,
                                                             const int* __restrict__ blocks) {
+  constexpr int V = 1;
   extern __shared__ double stein_sh[];
   double* fa = stein_sh;
   double* fb = fa + (size_t)nfull * V;
@@ -1546,69 +1491,7 @@ __global__ void __launch_bounds__(STEIN_THREADS) k_stein_sm(int nfull, const dou
     for (int w = 1; w < STEIN_THREADS / 32; ++w) tn = fmax(tn, sh_max[w][tid]);
     sh_tol[tid] = fmax(DBL_EPSILON * tn, DBL_MIN);
   }
-  // ---- elimination with partial pivoting
-  if (warp == 0) {
-    const int v = (lane >> 2) % V, sub = lane & 3;   // lanes past 4 V repeat the first vectors, unstored
-    const bool mine = lane < 4 * V && sub == 0;
-    const int n = sh_n[v];
-    const double* d = dfull + sh_s0[v];
-    const double* e = efull + sh_s0[v];
-    const double lam = sh_lam[v];
-    double ak = (n > 0) ? d[0] - lam : 1.0;
-    double bk = (n > 1) ? e[0] : 0.0;
-    double ck = bk, dn = (n > 1) ? d[1] : 0.0, en = (n > 2) ? e[1] : 0.0;
-    for (int k = 0; k + 1 < nmax; ++k) {
-      const bool on = k + 1 < n;
-      const double ak1 = dn - lam;
-      const double bk1 = en;                               // 0 from row n - 2 on
-      const double ckn = en;
-      dn = (k + 2 < n) ? d[k + 2] : 0.0;                   // next step's entries on their way
-      en = (k + 3 < n) ? e[k + 2] : 0.0;
-      const double scale1 = fabs(ak) + fabs(bk);
-      const double scale2 = fabs(ck) + fabs(ak1) + fabs(bk1);
-      const double num = (sub == 0) ? fabs(ak) : (sub == 1) ? fabs(ck) : (sub == 2) ? ck : ak;
-      const double den = (sub == 0) ? scale1 : (sub == 1) ? scale2 : (sub == 2) ? ak : ck;
-      const double q = num / den;
-      const int b4 = lane & ~3;
-      const double q0 = __shfl_sync(0xffffffffu, q, b4), piv2 = __shfl_sync(0xffffffffu, q, b4 + 1);
-      const double q2 = __shfl_sync(0xffffffffu, q, b4 + 2), q3 = __shfl_sync(0xffffffffu, q, b4 + 3);
-      const double piv1 = (scale1 == 0.0) ? 0.0 : q0;
-      if (on) {
-        double oa = ak, ob = bk, oc = 0.0, od = 0.0, na, nb = bk1;
-        unsigned char fl = 0;
-        if (ck == 0.0) {
-          na = ak1;
-        } else if (piv2 <= piv1) {
-          oc = q2;
-          na = ak1 - q2 * bk;
-        } else {
-          fl = 1;
-          oa = ck;
-          ob = ak1;
-          oc = q3;
-          na = bk - q3 * ak1;
-          if (k + 2 < n) {
-            od = bk1;
-            nb = -q3 * bk1;
-          } else {
-            nb = 0.0;
-          }
-        }
-        if (mine) {
-          const size_t x = (size_t)k * V + v;
-          fa[x] = oa;
-          fb[x] = ob;
-          fc[x] = oc;
-          fd[x] = od;
-          ff[x] = fl;
-        }
-        ak = na;
-        bk = nb;
-        ck = ckn;
-      }
-    }
-    if (mine && n > 0) fa[(size_t)(n - 1) * V + v] = ak;
-  }
+  if (warp == 0) stein_eliminate<V>(lane, nmax, sh_s0, sh_n, sh_lam, dfull, efull, fa, fb, fc, fd, ff);
   __syncthreads();
   // reciprocal pivots (tiny pivots replaced by +-tol)
   for (int x = tid; x < nmax * V; x += STEIN_THREADS) {
@@ -1642,7 +1525,10 @@ __global__ void __launch_bounds__(STEIN_THREADS) k_stein_sm(int nfull, const dou
         }
         fy[(size_t)(n - 1) * V + v] = yp;
       }
-      // backward; see k_stein for the rescaling
+      // backward: U^{-1}.  Each tiny pivot multiplies by up to 1/tol, so a cluster of
+      // them can overflow: whenever an entry passes 2^400 the whole vector (solved part
+      // and remaining right-hand side alike) is scaled by 2^-400, which keeps the system
+      // consistent; the vector is normalised afterwards anyway.
       unsigned long long ymax = 0ull;
       double y1 = 0.0, y2 = 0.0;
       double a = fa[(size_t)(n - 1) * V + v], b = 0.0, d2 = 0.0, yk0 = yp;
@@ -1683,6 +1569,209 @@ __global__ void __launch_bounds__(STEIN_THREADS) k_stein_sm(int nfull, const dou
       const int v = lane, n = sh_n[v];
       double nrm = 0.0;
 #pragma unroll 8
+      for (int k = 0; k < n; ++k) {
+        const double yk = fy[(size_t)k * V + v];
+        nrm = fma(yk, yk, nrm);
+      }
+      sh_sc[v] = 1.0 / sqrt(nrm);
+    }
+    __syncthreads();
+    for (int x = tid; x < nmax * V; x += STEIN_THREADS)
+      if (x / V < sh_n[x % V]) fy[x] *= sh_sc[x % V];
+    __syncthreads();
+  }
+#pragma unroll
+  for (int v = 0; v < V; ++v) {
+    if (t0 + v >= cnt) break;
+    double* out = Eout + (size_t)(t0 + v) * ldE;
+    const int s0 = sh_s0[v], n = sh_n[v];
+    for (int k = tid; k < nfull; k += STEIN_THREADS)
+      out[k] = (k >= s0 && k < s0 + n) ? fy[(size_t)(k - s0) * V + v] : 0.0;
+  }
+}
+
+// Working arrays in global memory: eight vectors per block, whose warp 0 serves them
+// side by side, and the chains load some entries ahead.
+__global__ void __launch_bounds__(STEIN_THREADS) k_stein_gl(int nfull, const double* __restrict__ dfull,
+                                                            const double* __restrict__ efull,
+                                                            const double* __restrict__ wsel, int cnt,
+                                                            double* __restrict__ Eout, int ldE, int tbase,
+                                                            const int* __restrict__ src,
+                                                            const int* __restrict__ blocks, double* ws) {
+  constexpr int V = STEIN_GL_V, CF = 8, CB = 4;   // entries on their way in the chains
+  double* fa = ws + (size_t)blockIdx.x * nfull * (5 * V + 1);
+  double* fb = fa + (size_t)nfull * V;
+  double* fc = fb + (size_t)nfull * V;
+  double* fd = fc + (size_t)nfull * V;
+  double* fy = fd + (size_t)nfull * V;
+  unsigned char* ff = reinterpret_cast<unsigned char*>(fy + (size_t)nfull * V);
+  __shared__ int sh_s0[V], sh_n[V];
+  __shared__ double sh_lam[V], sh_tol[V], sh_sc[V];
+  __shared__ double sh_max[STEIN_THREADS / 32][V];
+  const int t0 = blockIdx.x * V, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (tid < V) {
+    const int t = t0 + tid;
+    int s0 = 0, s1 = (t < cnt) ? nfull : 0;
+    if (blocks && t < cnt) {
+      const int b = blocks[src[t]];
+      s0 = blocks[nfull + b];
+      s1 = blocks[2 * nfull + b];
+    }
+    sh_s0[tid] = s0;
+    sh_n[tid] = s1 - s0;
+    sh_lam[tid] = (t < cnt) ? wsel[t] : 0.0;
+  }
+  __syncthreads();
+  int nmax = 0;
+#pragma unroll
+  for (int v = 0; v < V; ++v) nmax = max(nmax, sh_n[v]);
+  // tol from the largest row sum; start vectors
+#pragma unroll
+  for (int v = 0; v < V; ++v) {
+    const int n = sh_n[v];
+    const double* d = dfull + sh_s0[v];
+    const double* e = efull + sh_s0[v];
+    double tn = 0.0;
+    for (int i = tid; i < n; i += STEIN_THREADS) {
+      const double r = fabs(d[i]) + (i > 0 ? fabs(e[i - 1]) : 0.0) + (i + 1 < n ? fabs(e[i]) : 0.0);
+      tn = fmax(tn, r);
+      fy[(size_t)i * V + v] = hash_unif(((unsigned long long)(tbase + t0 + v) << 32) ^ (unsigned long long)i);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) tn = fmax(tn, __shfl_xor_sync(0xffffffffu, tn, o));
+    if (lane == 0) sh_max[warp][v] = tn;
+  }
+  __syncthreads();
+  if (tid < V) {
+    double tn = sh_max[0][tid];
+    for (int w = 1; w < STEIN_THREADS / 32; ++w) tn = fmax(tn, sh_max[w][tid]);
+    sh_tol[tid] = fmax(DBL_EPSILON * tn, DBL_MIN);
+  }
+  if (warp == 0) stein_eliminate<V>(lane, nmax, sh_s0, sh_n, sh_lam, dfull, efull, fa, fb, fc, fd, ff);
+  __syncthreads();
+  // reciprocal pivots (tiny pivots replaced by +-tol)
+  for (int x = tid; x < nmax * V; x += STEIN_THREADS) {
+    const int v = x % V;
+    if (x / V >= sh_n[v]) continue;
+    double a = fa[x];
+    if (fabs(a) < sh_tol[v]) a = (a >= 0.0) ? sh_tol[v] : -sh_tol[v];
+    fa[x] = 1.0 / a;
+  }
+  __syncthreads();
+  for (int iter = 0; iter < 3; ++iter) {
+    // four lanes run each chain side by side (the same values and stores): they share a rescaling
+    if (warp == 0 && sh_n[lane % V] > 0) {
+      const int v = lane % V, n = sh_n[v];
+      // forward
+      double yp = fy[v];
+      {
+        double c[CF], y[CF];
+        bool f[CF];
+        auto load = [&](int k0, double* cc, double* yy, bool* fl) {
+#pragma unroll
+          for (int u = 0; u < CF; ++u) {
+            const int k = k0 + u;
+            const bool in = k < n;
+            cc[u] = in ? fc[(size_t)(k - 1) * V + v] : 0.0;
+            yy[u] = in ? fy[(size_t)k * V + v] : 0.0;
+            fl[u] = in && ff[(size_t)(k - 1) * V + v] != 0;
+          }
+        };
+        load(1, c, y, f);
+        for (int k0 = 1; k0 < n; k0 += CF) {
+          double cn[CF], yn[CF];
+          bool fn[CF];
+          load(k0 + CF, cn, yn, fn);
+#pragma unroll
+          for (int u = 0; u < CF; ++u) {
+            const int k = k0 + u;
+            if (k >= n) break;
+            const double keep = f[u] ? y[u] : yp, other = f[u] ? yp : y[u];
+            fy[(size_t)(k - 1) * V + v] = keep;
+            yp = other - c[u] * keep;
+          }
+#pragma unroll
+          for (int u = 0; u < CF; ++u) {
+            c[u] = cn[u];
+            y[u] = yn[u];
+            f[u] = fn[u];
+          }
+        }
+        fy[(size_t)(n - 1) * V + v] = yp;
+      }
+      // backward
+      unsigned long long ymax = 0ull;
+      double y1 = 0.0, y2 = 0.0;
+      double a[CB], b[CB], d2[CB], y[CB];
+      auto load = [&](int k0, double* aa, double* bb, double* dd, double* yy) {
+#pragma unroll
+        for (int u = 0; u < CB; ++u) {
+          const int k = k0 - u;
+          const size_t x = (size_t)max(k, 0) * V + v;
+          aa[u] = fa[x];
+          bb[u] = (k + 1 < n) ? fb[x] : 0.0;
+          dd[u] = (k + 1 < n) ? fd[x] : 0.0;
+          yy[u] = fy[x];
+        }
+      };
+      load(n - 1, a, b, d2, y);
+      for (int k0 = n - 1; k0 >= 0; k0 -= CB) {
+        double an[CB], bn[CB], dn[CB], yn[CB];
+        load(k0 - CB, an, bn, dn, yn);
+#pragma unroll
+        for (int u = 0; u < CB; ++u) {
+          const int k = k0 - u;
+          if (k < 0) break;
+          double tmp = y[u];
+          if (k + 1 < n) tmp -= b[u] * y1;
+          if (k + 2 < n) tmp -= d2[u] * y2;
+          double yk = tmp * a[u];
+          if ((__double2hiint(yk) & 0x7FFFFFFF) >= 0x58F00000) {   // !(|yk| < 2^400)
+            const unsigned four = 0x01010101u << v;
+            __syncwarp(four);
+            for (int j0 = lane / V; j0 < n; j0 += 32) {
+              double z[8];
+#pragma unroll
+              for (int w = 0; w < 8; ++w) z[w] = (j0 + 4 * w < n) ? fy[(size_t)(j0 + 4 * w) * V + v] : 0.0;
+#pragma unroll
+              for (int w = 0; w < 8; ++w)
+                if (j0 + 4 * w < n) fy[(size_t)(j0 + 4 * w) * V + v] = z[w] * 0x1p-400;
+            }
+            __syncwarp(four);
+#pragma unroll
+            for (int w = 0; w < CB; ++w) {
+              y[w] *= 0x1p-400;
+              yn[w] *= 0x1p-400;
+            }
+            y1 *= 0x1p-400;
+            ymax = (unsigned long long)__double_as_longlong(__longlong_as_double((long long)ymax) * 0x1p-400);
+            yk = (tmp * 0x1p-400) * a[u];
+          }
+          fy[(size_t)k * V + v] = yk;
+          const unsigned long long q = (unsigned long long)__double_as_longlong(yk) & 0x7FFFFFFFFFFFFFFFull;
+          if (q <= 0x7FF0000000000000ull && q > ymax) ymax = q;
+          y2 = y1;
+          y1 = yk;
+        }
+#pragma unroll
+        for (int u = 0; u < CB; ++u) {
+          a[u] = an[u];
+          b[u] = bn[u];
+          d2[u] = dn[u];
+          y[u] = yn[u];
+        }
+      }
+      const double ym = __longlong_as_double((long long)ymax);
+      if (lane < V) sh_sc[v] = (ym > 0.0) ? 1.0 / ym : 1.0;
+    }
+    __syncthreads();
+    for (int x = tid; x < nmax * V; x += STEIN_THREADS)
+      if (x / V < sh_n[x % V]) fy[x] = fy[x] * sh_sc[x % V];
+    __syncthreads();
+    if (warp == 0 && lane < V) {
+      const int v = lane, n = sh_n[v];
+      double nrm = 0.0;
+#pragma unroll 16
       for (int k = 0; k < n; ++k) {
         const double yk = fy[(size_t)k * V + v];
         nrm = fma(yk, yk, nrm);
@@ -2040,42 +2129,31 @@ static void eigenvalues_all(cudaStream_t st, int n, EigWork* w, int nblocks, dou
   k_rank<<<cdiv(n, 128), 128, 0, st>>>(n, w->val, wout, w->src);
 }
 
-template <int V>
-static void launch_stein_sm(cudaStream_t st, int n, EigWork* w, const double* e, const double* wv, int first, int cnt,
-                            double* E, bool blk) {
-  allow_max_smem((const void*)k_stein_sm<V>);
-  count_launch();
-  k_stein_sm<V><<<cdiv(cnt, V), STEIN_THREADS, stein_sm_bytes(n, V), st>>>(
-      n, w->d, e, wv + first, cnt, E, n, first, blk ? w->src + first : nullptr, blk ? w->blocks : nullptr);
-}
-
-// Vectors per block of the shared-memory form: enough to keep the blocks to about
-// one per SM, as many as fit (8 up to order 670, 1 up to 5300).  It takes about
-// 1.75 us per unit of n and wave of blocks, the global-memory form about 8 us per
-// unit of n for any number of vectors, so from five waves on (n = 2000 with all its
-// vectors: seven waves, 24.7 ms against 19.2 ms) the latter runs.
+// The shared-memory form takes a vector per block, whose chain fills a scheduler: for up
+// to four blocks per SM (as many as there are schedulers, or as fit; n = 565, one vector
+// 0.99 ms against 1.31 ms, all of them 1.05 for both; n = 2000, one vector 3.5 against
+// 4.7).  More vectors, and orders above 5300, go eight to a block (n = 1000, all of them:
+// 1.9 ms, in shared memory 3.6).
 static void eigenvectors(cudaStream_t st, int n, EigWork* w, int nblocks, const double* wv, int first, int cnt,
                          double* E) {
   const double* e = (nblocks <= 1) ? w->e : w->es;
   const bool blk = nblocks > 1;
-  const size_t most = 220 * 1024;
-  int V = 8;
-  while (V > 1 && (stein_sm_bytes(n, V) > most || cnt <= 148 * (V / 2))) V /= 2;
-  const size_t need = stein_sm_bytes(n, V);
-  if (need <= most && cdiv(cnt, V) <= 4 * 148 * (most / need)) {
-    switch (V) {
-      case 8: launch_stein_sm<8>(st, n, w, e, wv, first, cnt, E, blk); break;
-      case 4: launch_stein_sm<4>(st, n, w, e, wv, first, cnt, E, blk); break;
-      case 2: launch_stein_sm<2>(st, n, w, e, wv, first, cnt, E, blk); break;
-      default: launch_stein_sm<1>(st, n, w, e, wv, first, cnt, E, blk); break;
-    }
+  const size_t need = stein_sm_bytes(n), most = 220 * 1024;
+  if (need <= most && cnt <= 148 * (int)std::min<size_t>(4, most / need)) {
+    allow_max_smem((const void*)k_stein_sm);
+    count_launch();
+    k_stein_sm<<<cnt, STEIN_THREADS, need, st>>>(n, w->d, e, wv + first, cnt, E, n, first,
+                                                              blk ? w->src + first : nullptr, blk ? w->blocks : nullptr);
     return;
   }
-  for (int t0 = 0; t0 < cnt; t0 += w->batch) {
-    const int c = std::min(w->batch, cnt - t0);
+  // blocks whose 5 V + 1 doubles per entry fit in the workspace of 6 per vector
+  const int batch = (int)(6ll * w->batch / (5 * STEIN_GL_V + 1)) * STEIN_GL_V;
+  for (int t0 = 0; t0 < cnt; t0 += batch) {
+    const int c = std::min(batch, cnt - t0);
     count_launch();
-    k_stein<<<cdiv(c, 64), 64, 0, st>>>(n, w->d, e, wv + first + t0, c, w->ws, w->batch, E + (size_t)t0 * n, n,
-                                        first + t0, blk ? w->src + first + t0 : nullptr, blk ? w->blocks : nullptr);
+    k_stein_gl<<<cdiv(c, STEIN_GL_V), STEIN_THREADS, 0, st>>>(n, w->d, e, wv + first + t0, c, E + (size_t)t0 * n, n,
+                                                              first + t0, blk ? w->src + first + t0 : nullptr,
+                                                              blk ? w->blocks : nullptr, w->ws);
   }
 }
 

@@ -118,3 +118,19 @@ def test_step_length_is_close_to_the_boundary(n):
     D = np.linalg.solve(L, np.linalg.solve(L, (X1 - X) / a).T)
     amax = -1.0 / np.linalg.eigvalsh((D + D.T) / 2)[0]
     assert 0.9 * 0.998 * amax * (1 - 1e-7) <= a <= 0.9 * amax * (1 + 1e-7)
+
+
+@pytest.mark.parametrize("n", [48, 606])
+def test_nt_scaling_of_block_matrices(n):
+    """Diagonal blocks of order 6: the tridiagonal form falls apart, every vector works on its own
+    block, with one vector per CTA (48) and with eight (606)."""
+    rng = np.random.default_rng(n)
+    X, S = np.zeros((n, n)), np.zeros((n, n))
+    for b in range(0, n, 6):   # spectra that differ from block to block
+        X[b:b + 6, b:b + 6] = _spectrum(6, rng.uniform(0.5, 2.0, 6), b)
+        S[b:b + 6, b:b + 6] = _spectrum(6, rng.uniform(0.5, 2.0, 6), b + 1)
+    with _prob(si.unit_diag_instance(n)) as prob:
+        prob.set_state(X, np.zeros(n), S, 0)
+        prob.ipm_step()
+        W = prob.get_W().cpu().numpy()
+    assert np.linalg.norm(W @ S @ W - X) <= 50 * n * EPS * 16.0 * np.linalg.norm(X)
