@@ -946,6 +946,159 @@ __global__ void __launch_bounds__(SYL_THREADS, 1) k_sytrd_cluster_lower(int n, d
   cluster.sync();   // no CTA leaves while another may still write into its shared memory
 }
 
+// One-triangle form for orders up to SYT_MAX_N: the same sums in the same order by one
+// CTA.  Warp r forms the column parts of the rows i = r mod 16 (CTA r's in the
+// cluster form), a row's dot and the sum of its 16 column parts take four lanes, warp 0
+// the sums over all rows and the next reflector while the others update.  Bound by the
+// chain of FP64 instructions of a column; the cluster form waits for two cluster barriers
+// and three remote accesses as well.  n = 40: 224 -> 169 us.
+constexpr int SYT_MAX_N = 64, SYT_LD = SYT_MAX_N + 1, SYT_THREADS = 512;
+__global__ void __launch_bounds__(SYT_THREADS) k_sytrd_small(int n, double* A, int lda, double* d, double* e,
+                                                             double* tauh) {
+  __shared__ double a[SYT_MAX_N * SYT_LD], part[16][SYT_MAX_N], sv[2][SYT_MAX_N], sw[SYT_MAX_N], p[SYT_MAX_N];
+  __shared__ double s_tau, s_beta;
+  const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31;
+  for (int t = tid; t < n * n; t += SYT_THREADS) {
+    const int i = t / n, c = t - i * n;
+    if (c <= i) a[i * SYT_LD + c] = __ldcg(A + (size_t)i * lda + c);
+  }
+  // Warp 0: the reflector of x (lane holds x0 = x[lane], x1 = x[lane + 32], m entries),
+  // its vector to v
+  auto reflector = [&](double x0, double x1, int m, double* v) {
+    double s = (lane > 0 && lane < m) ? fma(x0, x0, 0.0) : 0.0;
+    s += __shfl_xor_sync(0xffffffffu, s, 16);
+    if (m > 32) {
+      double s1 = (lane + 32 < m) ? fma(x1, x1, 0.0) : 0.0;
+      s1 += __shfl_xor_sync(0xffffffffu, s1, 16);
+      if (lane >= 16) s = s1;      // entries 32 and on in the upper lanes
+    }
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (m > 32) s = __shfl_sync(0xffffffffu, s, 0) + __shfl_sync(0xffffffffu, s, 16);
+    const double xf = __shfl_sync(0xffffffffu, x0, 0);
+    double tau = 0.0, beta = xf, scale = 0.0;
+    if (s > 0.0) {
+      beta = -copysign(sqrt(fma(xf, xf, s)), xf);
+      const double q = (lane == 1 ? 1.0 : beta - xf) / (lane == 1 ? xf - beta : beta);
+      tau = __shfl_sync(0xffffffffu, q, 0);
+      scale = __shfl_sync(0xffffffffu, q, 1);
+    }
+    if (lane == 0) {
+      s_tau = tau;
+      s_beta = beta;
+    }
+    if (lane < m) v[lane] = (lane == 0) ? 1.0 : x0 * scale;
+    if (lane + 32 < m) v[lane + 32] = x1 * scale;
+  };
+  __syncthreads();
+  if (wid == 0) {
+    const int m = n - 1;
+    reflector(lane < m ? a[(lane + 1) * SYT_LD] : 0.0, lane + 32 < m ? a[(lane + 33) * SYT_LD] : 0.0, m, sv[0]);
+  }
+  __syncthreads();
+  for (int j = 0; j < n - 2; ++j) {
+    const int len = n - j - 1;
+    const double* v = sv[j & 1];
+    const double tau = s_tau, beta = s_beta;
+    // ---- 1: column parts; row dots
+    for (int l = lane; l < len; l += 32) {
+      const int c = j + 1 + l;
+      double acc = 0.0;
+      for (int i = (c >= wid) ? c + 16 - ((c - wid) & 15) : wid; i < n; i += 16)
+        acc = fma(a[i * SYT_LD + c], v[i - j - 1], acc);
+      part[wid][l] = acc;
+    }
+    const int li = (SYT_THREADS / 32 - 1 - wid) * 8 + (lane >> 2), q = lane & 3;   // row j + 1 + li
+    const bool rows = (li & ~7) < len;   // of the whole warp
+    double dot = 0.0;
+    if (rows) {
+      const int cnt = (li < len) ? li + 1 : 0;
+      const double* ri = a + (j + 1 + min(li, len - 1)) * SYT_LD + j + 1;
+      double f[8];
+#pragma unroll
+      for (int m = 0; m < 8; ++m) {
+        const int x = q + 4 * m;
+        f[m] = (x < cnt) ? fma(ri[x], v[x], 0.0) : 0.0;
+        if ((li | 7) >= 32) f[m] = (x + 32 < cnt) ? fma(ri[x + 32], v[x + 32], f[m]) : f[m];
+      }
+#pragma unroll
+      for (int m = 0; m < 4; ++m) f[m] += f[m + 4];
+      f[0] += f[2];
+      f[1] += f[3];
+      dot = f[0] + f[1];
+      dot += __shfl_xor_sync(0xffffffffu, dot, 2);
+      dot += __shfl_xor_sync(0xffffffffu, dot, 1);
+    }
+    __syncthreads();
+    // ---- 2: p
+    if (rows) {
+      const int r = min(li, len - 1);
+      double s = (part[q][r] + part[q + 8][r]) + (part[q + 4][r] + part[q + 12][r]);
+      s += __shfl_xor_sync(0xffffffffu, s, 2);
+      s += __shfl_xor_sync(0xffffffffu, s, 1);
+      if (li < len && q == 0) p[li] = (dot + (s + 0.0)) * tau;   // a sum of zeros is +0
+    }
+    __syncthreads();
+    // ---- 3: warp 0: p^T v by the cluster form's shares, w and the next column
+    double x0 = 0.0, x1 = 0.0;
+    if (wid == 0) {
+      const int r = lane & 15;
+      const int i0 = (j + 1 > r) ? j + 1 + ((r - j - 1) & 15) : r;   // first row of share r after j
+      double kq[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int l = i0 + 16 * u - j - 1;
+        kq[u] = 0.0;
+        if (16 * u < len) kq[u] = (l < len) ? fma(p[l], v[l], 0.0) : 0.0;
+      }
+      double kp = kq[0];
+      if (len > 32) kp = (kq[0] + kq[2]) + (kq[1] + kq[3]);
+      else if (len > 16) kp = kq[0] + kq[1];
+      double K = 0.0;
+#pragma unroll
+      for (int c = 0; c < 16; ++c) K += __shfl_sync(0xffffffffu, kp, c);
+      K *= 0.5 * tau;
+      const double w0 = p[0] - K * v[0];
+      auto next = [&](int l) {   // w[l], returns the updated entry of column j + 1 in row j + 1 + l
+        const double vl = v[l], wl = p[l] - K * vl;
+        sw[l] = wl;
+        return fma(-vl, w0, fma(-wl, 1.0, a[(j + 1 + l) * SYT_LD + j + 1]));
+      };
+      if (lane == 0) sw[0] = w0;
+      if (lane + 1 < len) x0 = next(lane + 1);
+      if (len > 33 && lane + 33 < len) x1 = next(lane + 33);
+    }
+    __syncthreads();
+    if (wid == 0 && j + 1 < n - 2) reflector(x0, x1, len - 1, sv[(j + 1) & 1]);
+    if ((wid & 3) != 0) {
+      for (int l0 = (wid >> 2) * 3 + (wid & 3) - 1; l0 < len; l0 += 12) {
+        double* ri = a + (j + 1 + l0) * SYT_LD;
+        const double vi = v[l0], wi = sw[l0];
+        for (int l = lane; l <= l0; l += 32) ri[j + 1 + l] = fma(-vi, sw[l], fma(-wi, v[l], ri[j + 1 + l]));
+        if (lane == 0) ri[j] = vi;
+      }
+      if (tid == 32) {
+        d[j] = a[j * SYT_LD + j];
+        e[j] = beta;
+        tauh[j] = tau;
+      }
+    }
+    __syncthreads();
+  }
+  if (tid == 0) {
+    d[n - 2] = a[(n - 2) * SYT_LD + n - 2];
+    e[n - 2] = a[(n - 1) * SYT_LD + n - 2];
+    tauh[n - 2] = 0.0;
+    d[n - 1] = a[(n - 1) * SYT_LD + n - 1];
+    e[n - 1] = 0.0;
+    tauh[n - 1] = 0.0;
+  }
+  for (int t = tid; t < n * n; t += SYT_THREADS) {
+    const int i = t / n, c = t - i * n;
+    A[(size_t)i * lda + c] = (c <= i) ? a[i * SYT_LD + c] : a[c * SYT_LD + i];
+  }
+}
+
 static size_t sytrd_lower_smem_bytes(int n, int cs) {
   size_t most = 0;   // packed rows of the rank that holds the most
   for (int rank = 0; rank < cs; ++rank) {
@@ -1080,12 +1233,21 @@ static int sytrd_blocks(int n, size_t smem) {
 // once the O(n^3) work needs the whole GPU).
 constexpr int SY_CLUSTER_MAX_N = 1024;
 
-// Order of preference: the one-triangle form in cluster shared memory
+// Order of preference: up to order 64 the one-CTA form of the one-triangle sums (64: 44 KB of
+// static shared memory, one column chunk of 32 lanes twice); the one-triangle form in cluster shared memory
 // (n <= 880); the full-row form (n <= 656, where the device cannot run the
 // first); the L2-streaming cluster form; above order 1024 the resident form, then the
 // cooperative grid form.  The one-triangle form also leaves more room on its 16 SMs
 // for the other problems' kernels of a batch.
 static sdp_status sytrd(cudaStream_t st, int n, double* A, EigWork* w) {
+  // one CTA forms the cluster form's sums, so it stands in for it only where that runs
+  if (n >= 3 && n <= SYT_MAX_N && sytrd_lower_cluster(n) == 16) {
+    count_launch();
+    ktimer_begin(st, "sytrd");
+    k_sytrd_small<<<1, SYT_THREADS, 0, st>>>(n, A, n, w->d, w->e, w->tauh);
+    ktimer_end(st, "sytrd", 4.0 / 3.0 * n * (double)n * n, 16.0 * n * (double)n);
+    return SDP_OK;
+  }
   if (n >= 3 && n <= SY_CLUSTER_MAX_N) {
     const int cs = sytrd_lower_cluster(n);
     if (cs > 0) {
