@@ -421,14 +421,6 @@ void to_f32(cudaStream_t st, size_t count, const double* x, float* y) {
   count_launch();
   k_to_f32<<<std::min<unsigned>(cdiv(count, 256), 8192), 256, 0, st>>>(count, x, y);
 }
-__global__ void k_to_bf16(size_t count, const double* x, __nv_bfloat16* y) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < count; i += (size_t)gridDim.x * blockDim.x)
-    y[i] = __float2bfloat16_rn((float)x[i]);
-}
-void to_bf16(cudaStream_t st, size_t count, const double* x, __nv_bfloat16* y) {
-  count_launch();
-  k_to_bf16<<<std::min<unsigned>(cdiv(count, 256), 8192), 256, 0, st>>>(count, x, y);
-}
 
 // ---------------------------------------------------------------------------
 // Reductions (deterministic: fixed partition, fixed summation order)

@@ -229,7 +229,6 @@ void zero_upper(cudaStream_t st, int n, double* A, int lda);
 void axpby(cudaStream_t st, size_t count, double a, const double* x, double b, const double* y,
            double* z);                                                 // z = a x + b y
 void to_f32(cudaStream_t st, size_t count, const double* x, float* y);
-void to_bf16(cudaStream_t st, size_t count, const double* x, __nv_bfloat16* y);
 
 // Deterministic reductions into device memory (two stages, fixed order).
 // out[0] = sum_i x_i y_i.

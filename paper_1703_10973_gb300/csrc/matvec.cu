@@ -208,6 +208,16 @@ __global__ void __launch_bounds__(256) k_spmm_wv_small(int n, const int4* __rest
   if (t < n) T[(size_t)r * n + row.x] = acc;
 }
 
+// Rows of the reduced-precision W_s and T: lp_ld(n) entries, and in each full block of 32
+// columns those of one lane of the gather (its columns mod 8) side by side, so that a
+// lane loads four of its terms at once.  The load pipe bounds the gather: with one term
+// per load a wavefront moved 32 bytes.  n = 5024, 631014 constraints, BF16: the product
+// 3.02 -> 2.12 ms; n = 593, FP32: 72 -> 70 us.  Every sum keeps its order.
+__host__ __device__ __forceinline__ int lp_ld(int n) { return (n + 3) & ~3; }
+__device__ __forceinline__ int lp_pos(int n, int c) {
+  return (c < (n & ~31)) ? (c & ~31) | ((c & 7) << 2) | ((c >> 3) & 3) : c;
+}
+
 // Reduced precision: the R values of W_s that one stored entry of V needs lie side by
 // side (column-major staging), read by vector loads; they bound the kernel, so bfloat16
 // copies are staged as they are (half the bytes, widened in registers: the same
@@ -265,7 +275,7 @@ __device__ __forceinline__ void spmm_lp_body(int blk, int n, const int4* __restr
 #pragma unroll
   for (int rr = 0; rr < R; ++rr)
     for (int c = threadIdx.x; c < n; c += blockDim.x)
-      fsh[c * RS + rr] = (r0 + rr < n) ? W[(size_t)(r0 + rr) * n + c] : (TW)0.f;
+      fsh[c * RS + rr] = (r0 + rr < n) ? W[(size_t)(r0 + rr) * lp_ld(n) + lp_pos(n, c)] : (TW)0.f;
   int t = spmm_slice(w, nw, 0) * 32 + lane;
   int4 row = (t < n) ? sellrow[t] : make_int4(0, 0, 0, 0);   // on its way during the staging
   __syncthreads();
@@ -314,7 +324,7 @@ __device__ __forceinline__ void spmm_lp_body(int blk, int n, const int4* __restr
     }
 #pragma unroll
     for (int rr = 0; rr < R; ++rr)
-      if (r0 + rr < n) T[(size_t)(r0 + rr) * n + cur.x] = acc[rr];
+      if (r0 + rr < n) T[(size_t)(r0 + rr) * lp_ld(n) + lp_pos(n, cur.x)] = acc[rr];
   }
 }
 template <typename TW, int R>
@@ -457,6 +467,20 @@ void batch_launch_matvec(cudaStream_t st, const BDesc* desc, const int* off_asm,
   if (nb_sddmm > 0) kb_sddmm<<<nb_sddmm, 256, 0, st>>>(desc, off_sddmm, N);
 }
 
+__device__ __forceinline__ void lp_load4(const float* p, float* w) {
+  const float4 x = *reinterpret_cast<const float4*>(p);
+  w[0] = x.x;
+  w[1] = x.y;
+  w[2] = x.z;
+  w[3] = x.w;
+}
+__device__ __forceinline__ void lp_load4(const __nv_bfloat16* p, float* w) {
+  const uint2 x = *reinterpret_cast<const uint2*>(p);
+  w[0] = __uint_as_float(x.x << 16);
+  w[1] = __uint_as_float(x.x & 0xFFFF0000u);
+  w[2] = __uint_as_float(x.y << 16);
+  w[3] = __uint_as_float(x.y & 0xFFFF0000u);
+}
 template <typename TW>
 __device__ __forceinline__ void sddmm_lp_body(int lb, int nb, int n, int m, const int* __restrict__ eptr,
                                               const int* __restrict__ ep, const int* __restrict__ eq,
@@ -477,19 +501,20 @@ __device__ __forceinline__ void sddmm_lp_body(int lb, int nb, int n, int m, cons
     const int p = on ? ep[e0 + t] : 0, q = on ? eq[e0 + t] : 0;
     float s = 0.f;
     if (on) {
-      const TW* wp = W + (size_t)p * n;
-      const float* tq = T + (size_t)q * n;
-      int l = gl;
-      for (; l + 3 * SDDMM_L < n; l += 4 * SDDMM_L) {
-        const float w0 = tof<TW>(wp[l]), w1 = tof<TW>(wp[l + SDDMM_L]), w2 = tof<TW>(wp[l + 2 * SDDMM_L]),
-                    w3 = tof<TW>(wp[l + 3 * SDDMM_L]);
-        const float t0 = tq[l], t1 = tq[l + SDDMM_L], t2 = tq[l + 2 * SDDMM_L], t3 = tq[l + 3 * SDDMM_L];
-        s = fmaf(w0, t0, s);
-        s = fmaf(w1, t1, s);
-        s = fmaf(w2, t2, s);
-        s = fmaf(w3, t3, s);
+      const TW* wp = W + (size_t)p * lp_ld(n);
+      const float* tq = T + (size_t)q * lp_ld(n);
+      const int full = n & ~31;
+#pragma unroll 2
+      for (int b = 4 * gl; b < full; b += 32) {   // columns 32 b' + gl, + 8, + 16, + 24
+        float w[4];
+        lp_load4(wp + b, w);
+        const float4 t4 = *reinterpret_cast<const float4*>(tq + b);
+        s = fmaf(w[0], t4.x, s);
+        s = fmaf(w[1], t4.y, s);
+        s = fmaf(w[2], t4.z, s);
+        s = fmaf(w[3], t4.w, s);
       }
-      for (; l < n; l += SDDMM_L) s = fmaf(tof<TW>(wp[l]), tq[l], s);
+      for (int l = full + gl; l < n; l += SDDMM_L) s = fmaf(tof<TW>(wp[l]), tq[l], s);
     }
     double v = (double)gsum_f(s);
     if (k > 0) {
@@ -585,7 +610,7 @@ __device__ __forceinline__ void split_R_part_body(int bx, int by, int n, int k, 
     if (q < n) {
 #pragma unroll 8
       for (int c = 0; c < cnt; ++c) {
-        const float w = tof<TW>(Ws[(size_t)(cb + c) * n + q]);
+        const float w = tof<TW>(Ws[(size_t)(cb + c) * lp_ld(n) + lp_pos(n, q)]);
 #pragma unroll
         for (int l = 0; l < 8; ++l)
           if (l < k) acc[l] = fmaf(g[c * 8 + l], w, acc[l]);
@@ -751,14 +776,21 @@ void batch_launch_matvec_lp(cudaStream_t st, const BDesc* desc, const int* off_g
   if (with_sddmm && nb_sddmm > 0) kb_sddmm_lp<<<nb_sddmm, 256, 0, st>>>(desc, off_sddmm, N);
 }
 
+__device__ __forceinline__ void lp_store(float* y, double x) { *y = (float)x; }
+__device__ __forceinline__ void lp_store(__nv_bfloat16* y, double x) { *y = __float2bfloat16_rn((float)x); }
+template <typename TW>
+__global__ void __launch_bounds__(256) k_lp_copy(int n, const double* __restrict__ W, TW* __restrict__ Wl) {
+  const int r = blockIdx.x;
+  for (int c = threadIdx.x; c < n; c += 256) lp_store(Wl + (size_t)r * lp_ld(n) + lp_pos(n, c), W[(size_t)r * n + c]);
+}
 // Reduced-precision copy of W, or of W_s when a preconditioner with top
 // eigenpairs is built (the split form); keyed so that a new W or a rebuilt
 // preconditioner refreshes it.
 sdp_status ensure_lowprec_W(sdp_problem* h, int prec) {
   const int n = h->n;
-  const size_t nn = (size_t)n * n;
+  const size_t nn = (size_t)n * n, nl = (size_t)n * lp_ld(n);
   if (prec != SDP_FP32 && prec != SDP_BF16) return SDP_OK;
-  if (!h->T32) SDP_TRY(h->allocT(&h->T32, nn));
+  if (!h->T32) SDP_TRY(h->allocT(&h->T32, nl));
   const bool split = h->pc_valid && h->kpc > 0 && h->Etop && h->KZ && h->kpc <= 8;
   const int64_t key = split ? h->pc_generation : -1;
   bool& valid = (prec == SDP_FP32) ? h->W32_valid : h->W16_valid;
@@ -778,11 +810,13 @@ sdp_status ensure_lowprec_W(sdp_problem* h, int prec) {
     }
   }
   if (prec == SDP_FP32) {
-    if (!h->W32) SDP_TRY(h->allocT(&h->W32, nn));
-    to_f32(st, nn, src, h->W32);
+    if (!h->W32) SDP_TRY(h->allocT(&h->W32, nl));
+    count_launch();
+    k_lp_copy<float><<<n, 256, 0, st>>>(n, src, h->W32);
   } else {
-    if (!h->W16) SDP_TRY(h->allocT(&h->W16, nn));
-    to_bf16(st, nn, src, h->W16);
+    if (!h->W16) SDP_TRY(h->allocT(&h->W16, nl));
+    count_launch();
+    k_lp_copy<__nv_bfloat16><<<n, 256, 0, st>>>(n, src, h->W16);
   }
   valid = true;
   have_key = key;
