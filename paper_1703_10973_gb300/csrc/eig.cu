@@ -1,20 +1,17 @@
 // FP64 symmetric eigensolver for Algorithm 1 step 1 (eig(W)), the NT scaling
 // (eig(L^T S L)) and the step-length test (lambda_min).
 //
-//  1. Householder tridiagonalisation A = Q T Q^T in one cooperative persistent
-//     kernel: per column, every CTA rebuilds the reflector from row j (cheap,
-//     no barrier), warps own rows for the symmetric matrix-vector product and the
-//     rank-2 update; two bounded grid barriers per column.
-//  2. Eigenvalues of T by bisection on Sturm counts (one thread per eigenvalue).
-//  3. Eigenvectors of T by inverse iteration with a pivoted tridiagonal LU (one
-//     thread per eigenvalue, interleaved workspace so that the per-thread
-//     sequential sweeps load coalesced).
+//  1. Householder tridiagonalisation A = Q T Q^T: one CTA (n <= 64), a 16-CTA cluster
+//     (its shared memory up to n ~ 880, through L2 up to 1024), the whole GPU with the
+//     matrix in registers and shared memory (up to 2048) or in HBM; bounded barriers.
+//  2. Eigenvalues of T by multisection on Sturm counts (one warp per eigenvalue).
+//  3. Eigenvectors of T by inverse iteration with a pivoted tridiagonal LU (one vector
+//     per CTA in shared memory, eight in global memory).
 //  4. Re-orthogonalisation of the eigenvector block by up to two Cholesky-QR
 //     passes (Gram matrix GEMM, Cholesky, triangular solve), which repair the
 //     loss of orthogonality of inverse iteration inside eigenvalue clusters; a
 //     pass whose Gram matrix is already the identity to 1e-12 stops there.
-//  5. Back-transformation by the stored reflectors (one warp per eigenvector,
-//     no inter-CTA communication).
+//  5. Back-transformation by the stored reflectors (no inter-CTA communication).
 #include <cstring>
 #include "internal.cuh"
 
