@@ -1750,7 +1750,12 @@ __global__ void __launch_bounds__(STEIN_THREADS) k_stein_sm(int nfull, const dou
 }
 
 // Working arrays in global memory: eight vectors per block, whose warp 0 serves them
-// side by side, and the chains load some entries ahead.
+// side by side, and the chains load some entries ahead.  Four lanes follow a vector's
+// chain with the same values, so that they can share a rescaling; the first of them
+// stores.  A chain overwrites the entries that it read a batch earlier, and nothing
+// keeps four lanes together by itself (the chains of a warp differ in length and in
+// their rescalings), so the four meet after every batch of loads -- before the first
+// of them stores over it -- and between the passes.
 __global__ void __launch_bounds__(STEIN_THREADS) k_stein_gl(int nfull, const double* __restrict__ dfull,
                                                             const double* __restrict__ efull,
                                                             const double* __restrict__ wsel, int cnt,
@@ -1818,9 +1823,10 @@ __global__ void __launch_bounds__(STEIN_THREADS) k_stein_gl(int nfull, const dou
   }
   __syncthreads();
   for (int iter = 0; iter < 3; ++iter) {
-    // four lanes run each chain side by side (the same values and stores): they share a rescaling
     if (warp == 0 && sh_n[lane % V] > 0) {
       const int v = lane % V, n = sh_n[v];
+      const unsigned four = 0x01010101u << v;   // the lanes of this chain
+      const bool stores = lane < V;
       // forward
       double yp = fy[v];
       {
@@ -1841,12 +1847,13 @@ __global__ void __launch_bounds__(STEIN_THREADS) k_stein_gl(int nfull, const dou
           double cn[CF], yn[CF];
           bool fn[CF];
           load(k0 + CF, cn, yn, fn);
+          __syncwarp(four);   // all four have read up to entry k0 + 2 CF - 1
 #pragma unroll
           for (int u = 0; u < CF; ++u) {
             const int k = k0 + u;
             if (k >= n) break;
             const double keep = f[u] ? y[u] : yp, other = f[u] ? yp : y[u];
-            fy[(size_t)(k - 1) * V + v] = keep;
+            if (stores) fy[(size_t)(k - 1) * V + v] = keep;
             yp = other - c[u] * keep;
           }
 #pragma unroll
@@ -1856,8 +1863,10 @@ __global__ void __launch_bounds__(STEIN_THREADS) k_stein_gl(int nfull, const dou
             f[u] = fn[u];
           }
         }
-        fy[(size_t)(n - 1) * V + v] = yp;
+        __syncwarp(four);   // a chain of one entry: all four have read it
+        if (stores) fy[(size_t)(n - 1) * V + v] = yp;
       }
+      __syncwarp(four);     // the forward pass is stored
       // backward
       unsigned long long ymax = 0ull;
       double y1 = 0.0, y2 = 0.0;
@@ -1877,6 +1886,7 @@ __global__ void __launch_bounds__(STEIN_THREADS) k_stein_gl(int nfull, const dou
       for (int k0 = n - 1; k0 >= 0; k0 -= CB) {
         double an[CB], bn[CB], dn[CB], yn[CB];
         load(k0 - CB, an, bn, dn, yn);
+        __syncwarp(four);   // all four have read down to entry k0 - 2 CB + 1
 #pragma unroll
         for (int u = 0; u < CB; ++u) {
           const int k = k0 - u;
@@ -1886,8 +1896,7 @@ __global__ void __launch_bounds__(STEIN_THREADS) k_stein_gl(int nfull, const dou
           if (k + 2 < n) tmp -= d2[u] * y2;
           double yk = tmp * a[u];
           if ((__double2hiint(yk) & 0x7FFFFFFF) >= 0x58F00000) {   // !(|yk| < 2^400)
-            const unsigned four = 0x01010101u << v;
-            __syncwarp(four);
+            __syncwarp(four);   // what the first has stored in this batch
             for (int j0 = lane / V; j0 < n; j0 += 32) {
               double z[8];
 #pragma unroll
@@ -1906,7 +1915,7 @@ __global__ void __launch_bounds__(STEIN_THREADS) k_stein_gl(int nfull, const dou
             ymax = (unsigned long long)__double_as_longlong(__longlong_as_double((long long)ymax) * 0x1p-400);
             yk = (tmp * 0x1p-400) * a[u];
           }
-          fy[(size_t)k * V + v] = yk;
+          if (stores) fy[(size_t)k * V + v] = yk;
           const unsigned long long q = (unsigned long long)__double_as_longlong(yk) & 0x7FFFFFFFFFFFFFFFull;
           if (q <= 0x7FF0000000000000ull && q > ymax) ymax = q;
           y2 = y1;
