@@ -382,17 +382,6 @@ struct sdp_problem {
   float* T32 = nullptr;
   __nv_bfloat16* W16 = nullptr;
   bool W32_valid = false, W16_valid = false;
-  // fixed-point form of the FP64 Hessian product (matvec_fx.cu; lazily allocated)
-  void* fx_mem = nullptr;
-  int2 *fxW = nullptr, *fxT = nullptr;
-  int4* fxE = nullptr;
-  int *fx_exW = nullptr, *fx_exT = nullptr, *fx_exV = nullptr;
-  bool fx_valid = false;   // fxW holds the current W
-  int fx_R = 0, fx_split = 0, fx_ngrp[2] = {0, 0};   // layout of V (fx_layout); fx_R == 0: not used
-  int2 fx_rng[2] = {};
-  size_t fx_len = 0;
-  int2* fx_grp = nullptr;
-  int *fx_rid = nullptr, *fx_place = nullptr;
   int64_t W32_key = -1, W16_key = -1;   // preconditioner generation of a split copy (-1: plain W)
   double* mv_G = nullptr;  // split matvec: (E V)^T, n x k
   float* mv_R = nullptr;   // Lambda (E V) W_s, k x n
@@ -503,14 +492,6 @@ void pool_free(void* p, cudaStream_t st);
 // Optional epilogue (PCG): *dot_out = v . Hv, after *pro_dst = *pro_src.
 sdp_status matvec_impl(sdp_problem* h, const double* v, double* Hv, int prec, double* dot_out = nullptr,
                        double* pro_dst = nullptr, const double* pro_src = nullptr);
-// matvec_fx.cu: the FP64 product in fixed point, used where fx_pays after fx_prepare
-// (which allocates on its first call and refreshes the limbs of a new W)
-void fx_layout(sdp_problem* h, const std::vector<int>& rowptr, const std::vector<int>& colidx,
-               const std::vector<int>& rowperm, std::vector<int2>& grp, std::vector<int>& rid, std::vector<int>& place);
-bool fx_pays(const sdp_problem* h);
-sdp_status fx_prepare(sdp_problem* h);
-void fx_matvec(sdp_problem* h, const double* v, double* Hv, double* dot_out = nullptr, double* pro_dst = nullptr,
-               const double* pro_src = nullptr);
 sdp_status ensure_lowprec_W(sdp_problem* h, int prec);
 // sparse helpers used by the IPM and the preconditioner (matvec.cu)
 void assemble_V(sdp_problem* h, const double* v, const double* scale, double* Vval);
@@ -525,7 +506,7 @@ sdp_status precond_build_impl(sdp_problem* h);
 sdp_status precond_apply_impl(sdp_problem* h, const double* r, double* z, int prec, double* dot_out = nullptr);
 // pcg.cu
 sdp_status pcg_impl(sdp_problem* h, const double* r, double* y, double rtol, int maxit, int prec,
-                    int* iters, double* relres, bool fx = false);
+                    int* iters, double* relres);
 // ipm.cu
 sdp_status ipm_alloc(sdp_problem* h);
 // Batched PCG pieces (one launch for all problems of a batch; block offsets per problem)
@@ -566,8 +547,6 @@ struct PcgSweeps {
   double rtol = 0, inner_fp64 = 0, inner_lp = 0, tr = 1, nr0sq = 0;
   int maxit = 0, prec = 0, sweeps = 1, sweep = 0, total = 0, budget = 0;
   bool finished = false, graph = false;
-  bool fx = false;       // FP64 sweeps multiply in fixed point where that pays (matvec_fx.cu)
-  bool fx_now = false;   // the running sweep does
   sdp_status result = SDP_ERR_MAXIT;
 };
 sdp_status pcg_sweeps_init(sdp_problem* h, PcgSweeps* S, const double* r, double* y, double rtol, int maxit,

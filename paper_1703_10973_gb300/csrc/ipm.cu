@@ -442,7 +442,7 @@ sdp_status ipm_phase_a(sdp_problem* h, IpmStepState* s, bool* done) {
   }
   const int fb0 = h->nt_fallbacks;
   ktimer_begin(st, "nt_scaling");
-  h->W32_valid = h->W16_valid = h->fx_valid = false;
+  h->W32_valid = h->W16_valid = false;
   SDP_TRY(nt_scaling(h));
   ktimer_end(st, "nt_scaling", 0.0, 0.0);
   inf.nt_fallback = h->nt_fallbacks - fb0;

@@ -178,13 +178,12 @@ static sdp_status pcg_alloc(sdp_problem* h) {
 // One PCG iteration on h->stream (the body of the device-side loop): four
 // launches plus those of the two operators, whose last kernels also form the
 // two inner products (p . Hp with the move rz <- rz_new, and r . z).
-static sdp_status pcg_body(sdp_problem* h, int prec, bool fx, cudaGraphConditionalHandle cond, bool use_cond) {
+static sdp_status pcg_body(sdp_problem* h, int prec, cudaGraphConditionalHandle cond, bool use_cond) {
   cudaStream_t st = h->stream;
   const int m = h->m;
   const unsigned g = std::min(cdiv(m, 256), 2048u);
   double* scal = h->scal;
-  if (fx) fx_matvec(h, h->pp, h->pq, scal + S_PQ, scal + S_RZ, scal + S_RZN);
-  else SDP_TRY(matvec_impl(h, h->pp, h->pq, prec, scal + S_PQ, scal + S_RZ, scal + S_RZN));
+  SDP_TRY(matvec_impl(h, h->pp, h->pq, prec, scal + S_PQ, scal + S_RZ, scal + S_RZN));
   count_launch();
   k_pcg_xr_check<<<g, 256, 0, st>>>(m, h->px, h->pr, h->pp, h->pq, scal, h->pcg_part, h->pcg_ticket, cond,
                                     use_cond ? 1 : 0);
@@ -200,8 +199,8 @@ static sdp_status pcg_body(sdp_problem* h, int prec, bool fx, cudaGraphCondition
 // Build (or reuse) the executable graph: one while-node whose body is one PCG
 // iteration; the loop runs on the device until the recursive residual meets the
 // tolerance or the iteration budget is spent, with no host round trip.
-static sdp_status pcg_graph(sdp_problem* h, int prec, bool fx) {
-  const int64_t key = h->pc_generation * 8 + prec + (fx ? 4 : 0);
+static sdp_status pcg_graph(sdp_problem* h, int prec) {
+  const int64_t key = h->pc_generation * 8 + prec;
   if (h->pcg_exec && h->pcg_key == key) return SDP_OK;
   if (h->pcg_exec) {
     cudaGraphExecDestroy(h->pcg_exec);
@@ -229,7 +228,7 @@ static sdp_status pcg_graph(sdp_problem* h, int prec, bool fx) {
   const int64_t l0 = t_launches;
   ktimer_pause(true);
   cudaError_t e = cudaStreamBeginCaptureToGraph(h->stream, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
-  sdp_status s = (e == cudaSuccess) ? pcg_body(h, prec, fx, cond, true) : SDP_ERR_CUDA;
+  sdp_status s = (e == cudaSuccess) ? pcg_body(h, prec, cond, true) : SDP_ERR_CUDA;
   cudaGraph_t out = nullptr;
   cudaError_t e2 = cudaStreamEndCapture(h->stream, &out);
   ktimer_pause(false);
@@ -258,13 +257,12 @@ static double read_scalar(sdp_problem* h, const double* dev) {
 // Start of one PCG run from x = 0 on rhs (precision prec): r = rhs, z = M r,
 // p = z, scalars initialised on the device.  *nr0sq = ||rhs||^2 (zero: nothing
 // to run).  The loop itself is run by the caller (pcg_run, or a batch).
-static sdp_status pcg_start(sdp_problem* h, const double* rhs, double rtol, int maxit, int prec, bool* fx, bool graph,
+static sdp_status pcg_start(sdp_problem* h, const double* rhs, double rtol, int maxit, int prec, bool graph,
                             double* nr0sq) {
   cudaStream_t st = h->stream;
   const int m = h->m;
   double* scal = h->scal;
-  *fx = *fx && prec == SDP_FP64 && fx_pays(h) && fx_prepare(h) == SDP_OK;
-  if (graph) SDP_TRY(pcg_graph(h, prec, *fx));
+  if (graph) SDP_TRY(pcg_graph(h, prec));
   else SDP_TRY(ensure_lowprec_W(h, prec));
   SDP_CK(h, cudaMemcpyAsync(h->pr, rhs, m * sizeof(double), cudaMemcpyDeviceToDevice, st));
   SDP_CK(h, cudaMemsetAsync(h->px, 0, m * sizeof(double), st));
@@ -284,7 +282,7 @@ static sdp_status pcg_start(sdp_problem* h, const double* rhs, double rtol, int 
 }
 
 // The loop on the handle's own stream: the device-side graph, or the host loop.
-static sdp_status pcg_run(sdp_problem* h, int prec, bool fx, bool graph) {
+static sdp_status pcg_run(sdp_problem* h, int prec, bool graph) {
   cudaStream_t st = h->stream;
   if (graph) {
     SDP_CK(h, cudaGraphLaunch(h->pcg_exec, st));
@@ -292,7 +290,7 @@ static sdp_status pcg_run(sdp_problem* h, int prec, bool fx, bool graph) {
   }
   double go = 1.0;
   while (go != 0.0) {
-    SDP_TRY(pcg_body(h, prec, fx, cudaGraphConditionalHandle{}, false));
+    SDP_TRY(pcg_body(h, prec, cudaGraphConditionalHandle{}, false));
     SDP_CK(h, cudaMemcpyAsync(&go, h->scal + S_GO, sizeof(double), cudaMemcpyDeviceToHost, st));
     SDP_CK(h, cudaStreamSynchronize(st));
   }
@@ -383,9 +381,8 @@ sdp_status pcg_sweep_begin(sdp_problem* h, PcgSweeps* S, bool graph, bool* run) 
   const int base = std::max(500, kk * (kk + 1) / 2 + 500);
   S->budget = std::max(1, std::min(S->maxit - S->total, base << std::min(S->sweep, 3)));
   S->graph = graph;
-  S->fx_now = S->fx;
-  SDP_TRY(pcg_start(h, h->pbest, S->prec == SDP_FP64 ? S->inner_fp64 : S->inner_lp, S->budget, S->prec, &S->fx_now,
-                    graph, &S->nr0sq));
+  SDP_TRY(pcg_start(h, h->pbest, S->prec == SDP_FP64 ? S->inner_fp64 : S->inner_lp, S->budget, S->prec, graph,
+                    &S->nr0sq));
   if (S->nr0sq == 0.0) {
     S->finished = true;       // zero residual: y is exact already
     S->result = SDP_OK;
@@ -450,16 +447,15 @@ sdp_status pcg_sweep_end(sdp_problem* h, PcgSweeps* S) {
 }
 
 static sdp_status pcg_impl_(sdp_problem* h, const double* r, double* y, double rtol, int maxit, int prec,
-                            int* iters, double* relres, bool fx) {
+                            int* iters, double* relres) {
   PcgSweeps S;
   SDP_TRY(pcg_sweeps_init(h, &S, r, y, rtol, maxit, prec));
-  S.fx = fx;
   const bool graph = h->prm.pcg_graph != 0;
   for (;;) {
     bool run = false;
     SDP_TRY(pcg_sweep_begin(h, &S, graph, &run));
     if (!run) break;
-    SDP_TRY(pcg_run(h, S.prec, S.fx_now, graph));
+    SDP_TRY(pcg_run(h, S.prec, graph));
     SDP_TRY(pcg_sweep_end(h, &S));
   }
   if (iters) *iters = S.total;
@@ -468,9 +464,9 @@ static sdp_status pcg_impl_(sdp_problem* h, const double* r, double* y, double r
 }
 
 sdp_status pcg_impl(sdp_problem* h, const double* r, double* y, double rtol, int maxit, int prec, int* iters,
-                    double* relres, bool fx) {
+                    double* relres) {
   ktimer_begin(h->stream, "pcg");
-  sdp_status s = pcg_impl_(h, r, y, rtol, maxit, prec, iters, relres, fx);
+  sdp_status s = pcg_impl_(h, r, y, rtol, maxit, prec, iters, relres);
   ktimer_end(h->stream, "pcg", 0.0, 0.0);
   return s;
 }

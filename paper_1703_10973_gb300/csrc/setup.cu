@@ -390,16 +390,6 @@ static sdp_status build(sdp_problem* h, int64_t nnzC, const int32_t* Ci, const i
   SDP_TRY(upload(h, &h->sellrow, sellrow));
   SDP_TRY(upload(h, &h->sellcol, sellcol));
   SDP_TRY(upload(h, &h->sellpos, sellpos));
-  {
-    std::vector<int2> grp;
-    std::vector<int> rid, place;
-    fx_layout(h, rowptr, colidx, rowperm, grp, rid, place);
-    if (h->fx_R) {
-      SDP_TRY(upload(h, &h->fx_grp, grp));
-      SDP_TRY(upload(h, &h->fx_rid, rid));
-      SDP_TRY(upload(h, &h->fx_place, place));
-    }
-  }
   SDP_TRY(h->allocT(&h->Vsell, sellcol.size()));
   SDP_TRY(h->allocT(&h->Vsell32, sellcol.size()));
   SDP_TRY(upload(h, &h->colidx, colidx));
@@ -500,7 +490,7 @@ extern "C" sdp_status sdp_set_W(sdp_problem* h, const double* W_dev) {
   if (!h || !W_dev) return SDP_ERR_ARG;
   SDP_CK(h, cudaMemcpyAsync(h->W, W_dev, (size_t)h->n * h->n * sizeof(double), cudaMemcpyDeviceToDevice, h->stream));
   h->have_W = true;
-  h->W32_valid = h->W16_valid = h->fx_valid = false;
+  h->W32_valid = h->W16_valid = false;
   h->pc_valid = false;
   return SDP_OK;
 }
@@ -567,22 +557,8 @@ extern "C" sdp_status sdp_precond_info(sdp_problem* h, double* tau, int* k) {
 // ---- thin wrappers over the implementations in the other translation units
 extern "C" sdp_status sdp_hessian_matvec(sdp_problem* h, const double* v_dev, double* Hv_dev, int prec) {
   if (!h || !v_dev || !Hv_dev) return SDP_ERR_ARG;
-  // The fixed-point form reads limbs of W made when W was set.  A graph that the caller
-  // captures reads W itself, so that a replay sees the W of its time (and nothing is
-  // allocated in a capture).
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
-  if (prec == SDP_FP64 && h->have_W && fx_pays(h)) {
-    if (cudaStreamIsCapturing(h->stream, &cap) != cudaSuccess) {
-      cap = cudaStreamCaptureStatusActive;
-      cudaGetLastError();
-    }
-  }
-  if (cap == cudaStreamCaptureStatusNone && fx_prepare(h) == SDP_OK) {
-    fx_matvec(h, v_dev, Hv_dev);
-  } else {
-    sdp_status s = matvec_impl(h, v_dev, Hv_dev, prec);
-    if (s != SDP_OK) return s;
-  }
+  sdp_status s = matvec_impl(h, v_dev, Hv_dev, prec);
+  if (s != SDP_OK) return s;
   SDP_CK(h, cudaGetLastError());
   return SDP_OK;
 }
@@ -618,7 +594,7 @@ extern "C" sdp_status sdp_pcg_solve(sdp_problem* h, const double* r_dev, double*
     sdp_status s = sdp_precond_build(h);
     if (s != SDP_OK) return s;
   }
-  return pcg_impl(h, r_dev, y_dev, rtol, maxit, prec, iters, relres, true);
+  return pcg_impl(h, r_dev, y_dev, rtol, maxit, prec, iters, relres);
 }
 
 extern "C" sdp_status sdp_ipm_step(sdp_problem* h, sdp_ipm_info* info) {
@@ -638,6 +614,6 @@ extern "C" sdp_status sdp_reset(sdp_problem* h) {
   h->chol_valid = false;
   h->have_W = false;
   h->pc_valid = false;
-  h->W32_valid = h->W16_valid = h->fx_valid = false;
+  h->W32_valid = h->W16_valid = false;
   return SDP_OK;
 }
