@@ -95,8 +95,9 @@ typedef struct {
   double inner_rtol_lp; /* PCG tolerance of one sweep whose matvec runs in FP32 or */
                         /* BF16 (the FP64 true residual refines it); 1e-4         */
   long long wait_cycles; /* bound of every device-side spin wait (the grid barriers */
-                        /* of the cooperative tridiagonalisation, n > 1024), in SM */
-                        /* clock cycles; a wait that runs out makes the call return */
+                        /* of the cooperative tridiagonalisation, n > 1024, and of */
+                        /* the step lengths' Lanczos, n >= 256), in SM clock       */
+                        /* cycles; a wait that runs out makes the call return      */
                         /* SDP_ERR_TIMEOUT and leaves the handle usable; 0 = 4e9   */
                         /* (about 2 s)                                             */
   int k_max;            /* adaptive split rank (Section V implementation notes):   */

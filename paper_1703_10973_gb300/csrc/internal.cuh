@@ -276,7 +276,8 @@ sdp_status eig_full(cudaStream_t st, int n, double* A, double* w, double* E, Eig
 // Smallest eigenvalue only (result in *lmin_dev, device).
 sdp_status eig_min(cudaStream_t st, int n, double* A, double* lmin_dev, EigWork* ws);
 // lanczos.cu: lambda_min of a dense symmetric matrix (one thread-block cluster);
-// out_dev[0..4] = estimate, Ritz value, residual bound, steps, converged flag
+// out_dev[0..4] = estimate, Ritz value, residual bound, steps, converged flag (-1: a
+// wait ran out)
 size_t lanczos_work_doubles(int n);
 // schur.cu: sparse factorisation of the Hhat core
 struct SchurPlanHost {
@@ -297,7 +298,7 @@ sdp_status tc_gemm(cudaStream_t st, int prec, int M, int N, int K, const double*
                    const double* B, int ldb, bool transB, double* C, int ldc, void* work, int* err_dev);
 bool lanczos_fits(int n);
 sdp_status lanczos_min(cudaStream_t st, int n, const double* M, const double* A2, const double* A3, int ldm,
-                       double rtol, double accept_above, double* work, double* out_dev);
+                       double rtol, double accept_above, double* work, double* out_dev, long long spin);
 // Smallest eigenvalue and the top-k eigenpairs (k <= SDP_K_MAX + 1): wtop[0..k) ascending
 // (= lambda_{n-k..n-1}), Etop rows = eigenvectors; *lmin_dev = lambda_0.
 sdp_status eig_extremes(cudaStream_t st, int n, double* A, int k, double* lmin_dev, double* wtop,

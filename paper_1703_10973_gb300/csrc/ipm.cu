@@ -131,12 +131,18 @@ static sdp_status max_step(sdp_problem* h, const double* Lf, const double* Linv,
   if (h->lz_work) {
     // lambda_min by Lanczos; only whether it lies above -step_frac matters for a full step
     const sdp_status ls = implicit
-        ? lanczos_min(st, n, Linv, D, LinvT, n, 1e-3, -h->prm.step_frac, h->lz_work, h->scal + R_LZ)
-        : lanczos_min(st, n, h->M2, nullptr, nullptr, n, 1e-3, -h->prm.step_frac, h->lz_work, h->scal + R_LZ);
+        ? lanczos_min(st, n, Linv, D, LinvT, n, 1e-3, -h->prm.step_frac, h->lz_work, h->scal + R_LZ,
+                      h->prm.wait_cycles)
+        : lanczos_min(st, n, h->M2, nullptr, nullptr, n, 1e-3, -h->prm.step_frac, h->lz_work, h->scal + R_LZ,
+                      h->prm.wait_cycles);
     if (ls == SDP_OK) {
       double o[5];
       SDP_CK(h, cudaMemcpyAsync(o, h->scal + R_LZ, 5 * sizeof(double), cudaMemcpyDeviceToHost, st));
       SDP_CK(h, cudaStreamSynchronize(st));
+      if (o[4] < 0.0) {
+        h->last_error = "step length: grid barrier timeout";
+        return SDP_ERR_TIMEOUT;
+      }
       if (o[4] != 0.0 && std::isfinite(o[0])) {
         lmin = o[0];
         have = true;

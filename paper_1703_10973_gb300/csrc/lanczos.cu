@@ -356,9 +356,11 @@ __global__ void __cluster_dims__(LZ_CS, 1, 1) __launch_bounds__(LZ_THREADS)
 // stored zeros are skipped.  The convergence test is a serial computation of tens
 // of microseconds, so an extra CTA runs it while the others go on; when it says
 // stop, the (at most six) steps done meanwhile are dropped.  Every wait is
-// bounded; one that runs out ends the kernel with "not converged".
+// bounded (`spin` cycles of the SM clock; for the testing CTA, without an arrival
+// at a barrier): when one runs out, all CTAs leave, and without an accepted
+// estimate out[4] = -1.
 // ---------------------------------------------------------------------------
-constexpr long long LZ_SPIN_CYCLES = 4000000000ll;
+constexpr long long LZ_SPIN_CYCLES = 4000000000ll;   // the default, about two seconds
 constexpr int LZ_CHECKS = LZ_MAXIT / LZ_CHECK + 2;
 struct LzCtl {                 // zeroed before the launch
   unsigned int arrived;        // grid barrier: arrivals so far
@@ -376,7 +378,7 @@ __device__ __forceinline__ void lz_st(int* p, int v) {
   asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 // All workers arrive; false when the wait ran out somewhere.
-__device__ bool lz_barrier(LzCtl* c, unsigned int target) {
+__device__ bool lz_barrier(LzCtl* c, unsigned int target, long long spin) {
   __shared__ int s_ok;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -386,7 +388,7 @@ __device__ bool lz_barrier(LzCtl* c, unsigned int target) {
     int ok = 1;
     while ((unsigned int)lz_ld(reinterpret_cast<const int*>(&c->arrived)) < target) {
       if (lz_ld(&c->fail)) { ok = 0; break; }
-      if (clock64() - t0 > LZ_SPIN_CYCLES) { lz_st(&c->fail, 1); ok = 0; break; }
+      if (clock64() - t0 > spin) { lz_st(&c->fail, 1); ok = 0; break; }
     }
     __threadfence();
     s_ok = ok;
@@ -412,7 +414,7 @@ __device__ __forceinline__ void lz_gemv(int n, const double* __restrict__ A, int
 __global__ void __launch_bounds__(LZ_THREADS)
     k_lanczos_grid(int n, const double* __restrict__ M, const double* __restrict__ A2, const double* __restrict__ A3,
                    int ldm, double rtol, double accept_above, double* __restrict__ buf, double* __restrict__ out,
-                   LzCtl* ctl) {
+                   LzCtl* ctl, long long spin) {
   extern __shared__ double sm[];
   double* q = sm;                   // n   current q
   double* wb = sm + n;              // n   product, then the next direction
@@ -435,18 +437,24 @@ __global__ void __launch_bounds__(LZ_THREADS)
     __shared__ int s_req;
     for (int ci = 0; ci < LZ_CHECKS; ++ci) {
       if (threadIdx.x == 0) {
-        const long long t0 = clock64();
-        int rq;
+        const int* arrivals = reinterpret_cast<const int*>(&ctl->arrived);
+        long long t0 = clock64();
+        int rq, seen = lz_ld(arrivals);
         while ((rq = lz_ld(&ctl->req[ci])) == 0) {
           if (lz_ld(&ctl->fail)) break;
-          if (clock64() - t0 > LZ_SPIN_CYCLES) { lz_st(&ctl->fail, 1); break; }
+          if (clock64() - t0 > spin) {
+            const int now = lz_ld(arrivals);
+            if (now == seen) { lz_st(&ctl->fail, 1); break; }
+            seen = now;
+            t0 = clock64();
+          }
         }
         s_req = rq;
       }
       __syncthreads();
       const int rq = s_req;
       if (rq == 0) {
-        if (threadIdx.x == 0) out[4] = 0.0;
+        if (threadIdx.x == 0) out[4] = -1.0;
         return;
       }
       const int steps = rq & 1023;
@@ -482,7 +490,7 @@ __global__ void __launch_bounds__(LZ_THREADS)
   unsigned int target = 0;
   auto sync = [&]() {
     target += (unsigned)G;
-    return lz_barrier(ctl, target);
+    return lz_barrier(ctl, target, spin);
   };
   double s = 0.0;
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
@@ -587,12 +595,13 @@ constexpr int LZ_GRID_MIN_N = 256;
 // control block of the whole-GPU form.
 size_t lanczos_work_doubles(int n) { return (size_t)LZ_CS * (LZ_MAXIT + 1) * n + 8; }
 
-// Launch on st; results land in out_dev[0..4] (device).
+// Launch on st; results land in out_dev[0..4] (device).  spin: bound of a device-side wait
+// in SM clock cycles (0: the default).
 // Operator M (A2 = A3 = nullptr) or M A2 A3.  Needs 6 n doubles of shared memory per CTA.
 bool lanczos_fits(int n) { return n >= 2 && 6 * (size_t)n * sizeof(double) <= 200 * 1024; }
 
 sdp_status lanczos_min(cudaStream_t st, int n, const double* M, const double* A2, const double* A3, int ldm,
-                       double rtol, double accept_above, double* work, double* out_dev) {
+                       double rtol, double accept_above, double* work, double* out_dev, long long spin) {
   const size_t smem = 6 * (size_t)n * sizeof(double);
   if (!lanczos_fits(n) || (A2 == nullptr) != (A3 == nullptr)) return SDP_ERR_UNSUPPORTED;
   allow_max_smem((const void*)k_lanczos_min);
@@ -607,9 +616,10 @@ sdp_status lanczos_min(cudaStream_t st, int n, const double* M, const double* A2
     const int G = std::min((n + LZ_THREADS / 32 - 1) / (LZ_THREADS / 32), sms - 1);
     LzCtl* ctl = reinterpret_cast<LzCtl*>(work + lanczos_work_doubles(n) - (sizeof(LzCtl) + 7) / 8);
     const size_t sg = 4 * (size_t)n * sizeof(double);
+    if (spin <= 0) spin = LZ_SPIN_CYCLES;
     allow_max_smem((const void*)k_lanczos_grid);
     if (cudaMemsetAsync(ctl, 0, sizeof(LzCtl), st) != cudaSuccess) return SDP_ERR_CUDA;
-    void* args[] = {&n, &M, &A2, &A3, &ldm, &rtol, &accept_above, &work, &out_dev, &ctl};
+    void* args[] = {&n, &M, &A2, &A3, &ldm, &rtol, &accept_above, &work, &out_dev, &ctl, &spin};
     count_launch();
     ktimer_begin(st, "lanczos");
     const cudaError_t e = cudaLaunchCooperativeKernel((void*)k_lanczos_grid, dim3(G + 1), dim3(LZ_THREADS), args, sg, st);
