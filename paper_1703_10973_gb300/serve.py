@@ -30,27 +30,57 @@ import threading
 import time
 from dataclasses import dataclass, field
 
+import numpy as np
 
-def estimate_bytes(n: int, m: int, k: int, r_side: int | None = None) -> int:
-    """Upper estimate of the device bytes of one resident problem (FP64, Hhat).
 
-    About 31 dense n x n FP64 arrays (iterate, NT scaling, step-length inverses,
-    eigensolver workspace), the two dense Schur-complement factors of order
-    r_side * k (r_side: rows outside the independent set; n / 2 when unknown),
-    O(n k) preconditioner vectors, O(m) PCG vectors and constraint structure,
-    and a fixed allowance.
+def estimate_bytes(n: int, m: int, k: int, r_side: int | None = None, entries: int | None = None,
+                   couplings: int | None = None) -> int:
+    """Upper estimate of the device bytes of one resident problem (Hhat core, any precision).
+
+    entries: stored entries of all constraints (m when unknown: one each);
+    couplings: ordered pairs of different rows that one constraint touches, over
+    all constraints (2 m when unknown).  Counted are
+    - 32 dense n x n FP64 arrays (iterate, NT scaling, step-length inverses,
+      eigensolver workspace, reduced-precision copies);
+    - the Schur complement of the core, its inverse and that one's transpose, of
+      order r_side * k (r_side: rows outside the independent set; n / 2 when
+      unknown), and its k x k blocks;
+    - vectors and partial sums of O(n), O(n k) and O(r_side k);
+    - per constraint the PCG and right-hand-side vectors, per entry its two places in
+      the pattern (CSR and the sliced layout with its values) and the lists of its
+      rows, per coupling its place in the pattern of K and its contribution;
+    - the padding of the sliced layout (32 rows of at most n places) and a fixed
+      allowance.
     """
+    e = m if entries is None else entries
+    c = 2 * m if couplings is None else couplings
     rk = (r_side if r_side is not None else (n + 1) // 2) * k
-    return int(8 * (31 * n * n + 2 * rk * rk + 8 * n * k + 1000 * n) + 220 * m + (8 << 20))
+    slots = 2 * e                                       # upper bound: entries off the diagonal count twice
+    kslots = min(c, n * (n - 1))                        # off the diagonal of K
+    dense = 8 * (32 * n * n + 3 * rk * rk)
+    vectors = 8 * (1700 * n + 200 * n * (k + 1) + 200 * rk + n * k * k)
+    pattern = 68 * slots + 28 * 32 * n + 16 * e + (20 + 8 * (k + 1)) * slots
+    core = 28 * (kslots + n) + 12 * (c + slots) + (8 * k * k + 12) * ((kslots + 1) // 2)
+    return int(dense + vectors + pattern + core + 128 * m + (8 << 20))
 
 
 def estimate_request_bytes(d) -> int:
-    """estimate_bytes for an SDPData; matrix-completion instances give their smaller side."""
+    """estimate_bytes for an SDPData; matrix-completion instances give their smaller side, of
+    other ones any row may lie outside the independent set (none without couplings)."""
     meta = getattr(d, "meta", None) or {}
     r_side = None
     if "p" in meta and "q" in meta:
         r_side = min(int(meta["p"]), int(meta["q"]))
-    return estimate_bytes(d.n, d.m, d.k, r_side)
+    Ak, Ai, Aj = (np.asarray(x) for x in (d.Ak, d.Ai, d.Aj))
+    if d.m < 1 or d.n < 1 or not Ak.shape == Ai.shape == Aj.shape:
+        return estimate_bytes(d.n, d.m, d.k, r_side)   # setup refuses it
+    # rows that a constraint touches: at most two per entry off the diagonal
+    rows = np.bincount(np.clip(Ak, 0, d.m - 1), weights=1.0 + (Ai != Aj), minlength=d.m)
+    rows = np.minimum(rows, d.n)
+    couplings = int((rows * (rows - 1.0)).sum())
+    if r_side is None:
+        r_side = d.n if couplings else 0
+    return estimate_bytes(d.n, d.m, d.k, r_side, len(Ak), couplings)
 
 
 @dataclass
