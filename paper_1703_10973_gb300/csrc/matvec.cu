@@ -423,9 +423,12 @@ __global__ void kb_assemble(const BDesc* __restrict__ desc, const int* __restric
                 D.lp ? D.Vval : nullptr, D.sellpos, D.lp ? nullptr : D.Vsell, D.lp ? D.Vsell32 : nullptr);
 }
 // R rows of W per CTA: chosen per batch by the autotuner (batch.cu); every R
-// gives each entry of T by the same sequence of FMAs, so results do not depend on it
+// gives each entry of T by the same sequence of FMAs, so results do not depend on it.
+// Two CTAs on an SM (64 registers a thread, no spills), so that one stages its rows of W
+// beside the other's multiply-adds.  16 problems of order 181 to 740, cold caches: 547 us
+// with R = 2; with one CTA an SM (77 registers for R = 4) 593 us.
 template <int R>
-__global__ void __launch_bounds__(512) kb_spmm(const BDesc* __restrict__ desc, const int* __restrict__ off, int N) {
+__global__ void __launch_bounds__(512, 2) kb_spmm(const BDesc* __restrict__ desc, const int* __restrict__ off, int N) {
   extern __shared__ double wsh[];
   const int i = batch_find(off, N, blockIdx.x);
   const BDesc& D = desc[i];
