@@ -144,7 +144,8 @@ __device__ __forceinline__ void spmm_f64_body(int blk, int n, const int4* __rest
 #pragma unroll
         for (int rr = 0; rr < R; ++rr) acc[rr] = fma(val[u], wsh[rr * n + col[u]], acc[rr]);
     }
-    if (s < len) {   // fewer than eight left
+    if (s < len) {   // fewer than eight left: loads together, an exit after the last (a
+                     // multiply-add that is predicated off would hold the FP64 pipe as well)
       int col[SPMM_UNROLL];
       double val[SPMM_UNROLL];
 #pragma unroll
@@ -154,11 +155,11 @@ __device__ __forceinline__ void spmm_f64_body(int blk, int n, const int4* __rest
           val[u] = vp[32 * (s + u)];
         }
 #pragma unroll
-      for (int u = 0; u < SPMM_UNROLL - 1; ++u)
-        if (s + u < len) {
+      for (int u = 0; u < SPMM_UNROLL - 1; ++u) {
+        if (s + u >= len) break;
 #pragma unroll
-          for (int rr = 0; rr < R; ++rr) acc[rr] = fma(val[u], wsh[rr * n + col[u]], acc[rr]);
-        }
+        for (int rr = 0; rr < R; ++rr) acc[rr] = fma(val[u], wsh[rr * n + col[u]], acc[rr]);
+      }
     }
 #pragma unroll
     for (int rr = 0; rr < R; ++rr)
@@ -174,11 +175,62 @@ __global__ void __launch_bounds__(512) k_spmm_wv_f64(int n, const int4* __restri
   spmm_f64_body<R>(blockIdx.x, n, sellrow, sellcol, Vsell, W, T, wsh);
 }
 
-// The product of small orders, where launches and latency count: the values of V are
-// formed where they are used (every slot has one contributor; the place's
-// constraint and coefficient lie in the sliced layout), so the assembly is no
-// launch of its own.  One row of W per CTA.  n = 40: 12.4 -> 9.9 us for the product.
-constexpr int SPMM_SMALL_N = 192;
+// One row of W per CTA and at most one row of V per thread (n <= SPMM_ONE_N): a few
+// warps per SM, bound by the latency of the entries' loads.  The first eight are on
+// their way during the staging and the next eight during the multiply-adds.  The whole
+// product, 75 x 75 with 2400 samples (n = 150): 11.3 us, with the loads of
+// spmm_f64_body 15.5; 152 x 152 with 11552: 27.9 and 29.3.
+constexpr int SPMM_ONE_N = 512;
+__global__ void __launch_bounds__(512) k_spmm_wv_one(int n, const int4* __restrict__ sellrow,
+                                                     const int* __restrict__ sellcol,
+                                                     const double* __restrict__ Vsell,
+                                                     const double* __restrict__ W, double* __restrict__ T) {
+  __shared__ double w[SPMM_ONE_N];
+  const int r = blockIdx.x, t = spmm_slice(threadIdx.x >> 5, blockDim.x >> 5, 0) * 32 + (threadIdx.x & 31);
+  const int4 row = (t < n) ? sellrow[t] : make_int4(0, 0, 0, 0);
+  for (int c = threadIdx.x; c < n; c += blockDim.x) w[c] = W[(size_t)r * n + c];
+  const int len = row.y;
+  const int* cp = sellcol + row.z;
+  const double* vp = Vsell + row.z;
+  int col[SPMM_UNROLL];
+  double val[SPMM_UNROLL];
+  auto load = [&](int s, int* cl, double* vl) {
+#pragma unroll
+    for (int u = 0; u < SPMM_UNROLL; ++u) {
+      cl[u] = (s + u < len) ? cp[32 * (s + u)] : 0;
+      vl[u] = (s + u < len) ? vp[32 * (s + u)] : 0.0;
+    }
+  };
+  load(0, col, val);
+  __syncthreads();
+  double acc = 0.0;
+  for (int s = 0; s < len; s += SPMM_UNROLL) {
+    int col1[SPMM_UNROLL];
+    double val1[SPMM_UNROLL];
+    load(s + SPMM_UNROLL, col1, val1);
+#pragma unroll
+    for (int u = 0; u < SPMM_UNROLL; ++u) {
+      if (s + u >= len) break;
+      acc = fma(val[u], w[col[u]], acc);
+    }
+#pragma unroll
+    for (int u = 0; u < SPMM_UNROLL; ++u) {
+      col[u] = col1[u];
+      val[u] = val1[u];
+    }
+  }
+  if (t < n) T[(size_t)r * n + row.x] = acc;
+}
+
+// The product of small orders and short rows, where launches and latency count: the
+// values of V are formed where they are used (every slot has one contributor; the
+// place's constraint and coefficient lie in the sliced layout), so the assembly is no
+// launch of its own.  One row of W per CTA.  An entry takes two dependent loads here, so
+// long rows lose more than the launch is worth.  In a graph, where only the device's
+// time counts, n = 100 with 4 / 8 / 12 / 24 entries per row takes 7.6 / 8.4 / 9.5 / 12.4
+// us against 7.8 / 8.2 / 8.3 / 9.1 for the assembly and k_spmm_wv_one; launched one by
+// one, n = 40 with 10 entries takes 10.3 us against 12.3.  The line lies at 12 entries.
+constexpr int SPMM_SMALL_N = 192, SPMM_SMALL_LEN = 12;
 __global__ void __launch_bounds__(256) k_spmm_wv_small(int n, const int4* __restrict__ sellrow,
                                                        const int* __restrict__ sellcol,
                                                        const int* __restrict__ sellcon,
@@ -202,8 +254,10 @@ __global__ void __launch_bounds__(256) k_spmm_wv_small(int n, const int4* __rest
       }
     if (s == 0) __syncthreads();
 #pragma unroll
-    for (int u = 0; u < SPMM_UNROLL; ++u)
-      if (s + u < row.y) acc = fma(val[u], w[col[u]], acc);
+    for (int u = 0; u < SPMM_UNROLL; ++u) {
+      if (s + u >= row.y) break;
+      acc = fma(val[u], w[col[u]], acc);
+    }
   }
   if (t < n) T[(size_t)r * n + row.x] = acc;
 }
@@ -872,7 +926,14 @@ static void spmm_f64(sdp_problem* h) {
     case 4: launch_spmm_f64<4>(h); break;
     case 3: launch_spmm_f64<3>(h); break;
     case 2: launch_spmm_f64<2>(h); break;
-    default: launch_spmm_f64<1>(h); break;
+    default:
+      if (h->n <= SPMM_ONE_N) {
+        count_launch();
+        k_spmm_wv_one<<<h->n, spmm_threads(h->n), 0, h->stream>>>(h->n, h->sellrow, h->sellcol, h->Vsell, h->W, h->T);
+      } else {
+        launch_spmm_f64<1>(h);
+      }
+      break;
   }
 }
 template <typename TW, int R>
@@ -905,7 +966,7 @@ sdp_status matvec_impl(sdp_problem* h, const double* v, double* Hv, int prec, do
   const bool timed = ktimer_on("matvec");
   if (timed) ktimer_begin(h->stream, "matvec");
   if (prec == SDP_FP64) {
-    if (h->sellcon && n <= SPMM_SMALL_N) {
+    if (h->sellcon && n <= SPMM_SMALL_N && h->nnzV <= SPMM_SMALL_LEN * n) {
       count_launch();
       k_spmm_wv_small<<<n, (n + 31) / 32 * 32, 0, h->stream>>>(n, h->sellrow, h->sellcol, h->sellcon, h->sellcoef, v,
                                                                h->W, h->T);
