@@ -328,8 +328,8 @@ struct sdp_problem {
   // The same entries for the SpMM (sliced ELL): slices of 32 rows by decreasing
   // length, entry j of a slice's 32 rows side by side, so that a warp whose lanes walk one
   // row each reads whole lines
-  int4* sellrow = nullptr; // n   row, length, first place, by decreasing length
-  int* sellcol = nullptr;  // column of every place (padding: 0, never read)
+  int4* sellrow = nullptr; // n   row, length, first place, by decreasing length (the start of one allocation)
+  int* sellcol = nullptr;  // column of every place (the padding is never read)
   int* sellpos = nullptr;  // nnzV   slot -> place
   int* sellcon = nullptr;  // constraint and coefficient of every place, where each slot has one contributor
   double* sellcoef = nullptr;
