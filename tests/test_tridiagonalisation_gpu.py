@@ -1,5 +1,6 @@
 """Tridiagonalisation above order 1024: the resident form up to 2048, beyond it the one that streams the
-matrix -- its results on both sides of that order, and a grid barrier's wait that runs out in either."""
+matrix -- its results on both sides of that order, a grid barrier's wait that runs out in either, and the
+step lengths, which need a factor of the iterate and the smallest eigenvalue only."""
 import numpy as np
 import pytest
 
@@ -80,3 +81,37 @@ def test_top_pairs_above_order_1024(n):
     np.add.at(V, j, 0.5 * z[:, None] * U[i])
     Hz = lo * lo * 0.5 * z + 2.0 * lo * 0.5 * ((V[i] * U[j]).sum(1) + (V[j] * U[i]).sum(1))
     assert np.linalg.norm(Hz - r) <= 4 * n * EPS * (1 + 2 * 60.0 / lo) * np.linalg.norm(r)
+
+
+@pytest.mark.parametrize("n", [1025, 2047])
+def test_nt_scaling_above_order_1024(n):
+    """All eigenvectors, back-transformed: W S W = X to 50 n eps kappa(X) kappa(S), kappa <= 4 each."""
+    from paper_1703_10973_gb300 import SDPProblem
+    rng = np.random.default_rng(n)
+    X, S = _spectrum(n, rng.uniform(0.5, 2.0, n), 1), _spectrum(n, rng.uniform(0.5, 2.0, n), 2)
+    with SDPProblem.from_data(si.unit_diag_instance(n)) as prob:
+        prob.set_state(X, np.zeros(n), S, 0)
+        info = prob.ipm_step()
+        W = prob.get_W().cpu().numpy()
+    assert info["nt_fallback"] == 0
+    assert np.linalg.norm(W @ S @ W - X) <= 50 * n * EPS * 16.0 * np.linalg.norm(X)
+
+
+@pytest.mark.parametrize("n", [63, 64, 255, 256, 257, 519, 1025])
+def test_step_that_the_boundary_cuts(n):
+    """X twenty times too large: the step to X_ii = 1 leaves the cone.  alpha = 0.9 / -(theta - bound)
+    with bound <= 1e-3 |theta| and theta - bound <= lambda_min(L^-1 dX L^-T) up to rounding: between
+    0.998 of 0.9 of the largest step and that, on both sides of the orders at which Lanczos changes."""
+    from paper_1703_10973_gb300 import SDPProblem
+    rng = np.random.default_rng(n)
+    U, V = (rng.standard_normal((n, 8)) / np.sqrt(n) for _ in range(2))
+    X, S = 20.0 * (0.7 * np.eye(n) + U @ U.T), 0.9 * np.eye(n) + V @ V.T
+    with SDPProblem.from_data(si.unit_diag_instance(n)) as prob:
+        prob.set_state(X, np.zeros(n), S, 0)
+        a = prob.ipm_step()["alpha_p"]
+        X1, _, _ = prob.get_solution()
+    assert a < 1.0
+    L = np.linalg.cholesky(X)
+    D = np.linalg.solve(L, np.linalg.solve(L, (X1 - X) / a).T)
+    amax = -1.0 / np.linalg.eigvalsh((D + D.T) / 2)[0]
+    assert 0.9 * 0.998 * amax * (1 - 1e-7) <= a <= 0.9 * amax * (1 + 1e-7)
