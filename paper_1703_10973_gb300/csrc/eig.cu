@@ -1588,7 +1588,7 @@ __device__ __forceinline__ void stein_eliminate(int lane, int nmax, const int* s
 // Bound by that serial chain of FP64 instructions (64 cycles of a scheduler's pipe
 // each).  Two forms with the same operations in the same order, for the working arrays
 // in shared memory and in global memory; a thread per vector through L2 took 4.2 ms at
-// n = 565, 22.8 ms at n = 2000 for all vectors, here 1.1 and 4.1 ms.
+// n = 565, 22.8 ms at n = 2000 for all vectors, here 1.1 and 4.2 ms.
 // Fields, index k, vector v at [(f n + k) V + v]: 0 a (reciprocal pivots), 1 b,
 // 2 c (multipliers), 3 d2, 4 y; then n V pivot flags.
 constexpr int STEIN_THREADS = 128;
@@ -2039,7 +2039,7 @@ __global__ void __launch_bounds__(256) k_ormtr_sm(int n, const double* __restric
   if (have)
     for (int l = lane; l < n; l += 32) E[(size_t)t * ldE + l] = x[l];
 }
-// Warps per block: about one block per SM; from 592 vectors on eight, so that every
+// Warps per block: about one block per SM (148 of the 152); from 592 vectors on eight, so that every
 // scheduler has a second warp to issue while one waits.  Orders whose working set
 // does not fit (above 2300 with eight warps, 3500 with four) run k_ormtr_rows.
 // All vectors and the top ones of a build together: n = 565 4.0 -> 1.8 ms, n = 2000

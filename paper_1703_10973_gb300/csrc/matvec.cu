@@ -730,9 +730,9 @@ __global__ void k_split_Ws(int n, int k, const double* __restrict__ W, const dou
 // Batched FP32 forms: the same bodies as the single-problem launches (problems
 // in an FP64 sweep return at once).  Each entry of T is one thread's sum in the
 // row's CSR order whatever the rows per CTA, so the batched SpMM may take more
-// rows of W per CTA than a problem alone and still match it bit for bit: 16 (a
-// quarter of the CSR re-reads of 4) while the staged rows of the batch's
-// largest problem fit in 200 KB of shared memory, fewer for larger orders.
+// rows of W per CTA than a problem alone and still match it bit for bit: 16 (V is
+// read n / 16 times) while the staged rows of the batch's largest problem fit in
+// 200 KB of shared memory, fewer for larger orders.
 int batch_spmm_lp_rows(int nmax) {
   for (int r = 16; r > 1; r /= 2)
     if (spmm_lp_bytes<float>(r) * nmax <= 200 * 1024) return r;

@@ -2,8 +2,9 @@
 //
 // An FP64 instruction holds a scheduler's pipe for 64 cycles on this GPU, so a
 // division or square root (ten to twenty of them in a row) takes 1000 cycles or
-// more -- most of the time of a serial step that needs one (a Cholesky pivot, a
-// Householder reflector, a pivot of a tridiagonal).  These versions use 64-bit
+// more.  The quotients of the two substitutions of the Hhat apply take div_rn; pivots of
+// Cholesky, reflectors and tridiagonal eliminations were no faster with it.  sqrt_rn
+// has no caller: it is kept with its test.  These versions use 64-bit
 // integer products: a 23-bit approximation from the FP32 unit, two Newton steps
 // in fixed point (62 bits), and the exact remainder, which decides the rounding to
 // nearest even.  IEEE rounding leaves one possible result, so they return what the
