@@ -398,9 +398,10 @@ def instrumented_step(args, insts, prec, kk, stream):
 
 
 # All-active batched FP64 matvec of the 16 bench instances: algorithmic flops
-# (2 nnz(V) n + 2 nent n summed) and the DRAM bytes ncu measured for its SpMM and SDDMM.
+# (2 nnz(V) n + 2 nent n summed) and the DRAM bytes ncu measured for its V assembly, SpMM
+# and SDDMM.
 MATVEC_B_ALL_ACTIVE_FLOPS = 0.558157e9 + 0.279079e9
-MATVEC_B_NCU_BYTES = 36.78e6 + 36.97e6
+MATVEC_B_NCU_BYTES = 10.85e6 + 36.30e6 + 36.91e6
 
 
 def roofline_of(cls, rep, wall):
@@ -526,12 +527,12 @@ def run(args):
         roof = rooflines.get(f"fp64:{want}") or next(iter(rooflines.values()), None)
         if roof is not None and roof["kernel"] == "matvec_b" and args.workload == "batched" and args.batch == 16:
             # DRAM bytes of one all-active batched matvec of these 16 instances (ncu
-            # captures: SpMM 36.8 MB, SDDMM 37.0 MB; the V assembly is not captured),
-            # scaled to the average launch by the flops it did
+            # captures: V assembly 10.8 MB, SpMM 36.3 MB, SDDMM 36.9 MB), scaled to the
+            # average launch by the flops it did
             t_all, f_all = MATVEC_B_NCU_BYTES, MATVEC_B_ALL_ACTIVE_FLOPS
             per_launch_flops = roof["achieved"] * 1e12 * roof["avg_us"] * 1e-6
             roof["traffic"] = t_all * per_launch_flops / f_all
-            roof["traffic_source"] = ("ncu dram__bytes_read.sum + dram__bytes_write.sum of kb_spmm + kb_sddmm with all "
+            roof["traffic_source"] = ("ncu dram__bytes_read.sum + dram__bytes_write.sum of kb_assemble + kb_spmm + kb_sddmm with all "
                                       "16 problems active (profiles/ncu_batched_spmm_16mc.md, "
                                       "profiles/ncu_batched_sddmm_16mc.md), scaled by the average launch's flops")
 
